@@ -766,7 +766,11 @@ demag_status create_plan(int nx, int ny, int nz, double dx, double dy, double dz
     p->prec = prec;
     p->Px = P[0]; p->Py = P[1]; p->Pz = P[2];
     p->Kx = P[0] == 1 ? 1 : P[0] / 2 + 1;
-    p->Kxp = P[0] == 1 ? 1 : (p->Kx + 1) / 2 * 2;
+    // rows start on 32-byte sectors: a 64-byte tile row of the y and z passes
+    // then touches two sectors instead of three (512 x 512 x 128: 3.10 -> 3.06 ms a
+    // field; whole 128-byte lines cost more memory traffic than they save: 3.12)
+    const int row_unit = prec == DEMAG_F32 ? 4 : 2;
+    p->Kxp = P[0] == 1 ? 1 : (p->Kx + row_unit - 1) / row_unit * row_unit;
     if (cudaGetDevice(&p->device) != cudaSuccess) {
         cudaGetLastError();
         delete p;
