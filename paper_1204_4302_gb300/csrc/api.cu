@@ -416,7 +416,8 @@ demag_status run_field(demag_plan *p, const FieldJob &job, cudaStream_t st)
     }
     if (e == cudaErrorNotSupported)
         e = Passes<T>::zconv(Pz, S2, Py * Kx, Kx, Kxp, (int64_t)Py * Kxp, (int64_t)nz * Py * Kxp, nz, nhat, Py, Kx,
-                             twz, 1, st, (p->zvariant == 6 || p->zvariant == 7) ? 0 : p->zvariant);
+                             twz, 1, st, (p->zvariant == 6 || p->zvariant == 7) ? 0 : p->zvariant,
+                             f32 ? (const T *)(const void *)p->ntile : nullptr);
     if (e != cudaSuccess) return fail(DEMAG_ERR_CUDA, std::string("z convolution: ") + cudaGetErrorString(e));
     p->launches++;
     tm.mark();

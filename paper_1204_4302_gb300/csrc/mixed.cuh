@@ -221,7 +221,7 @@ template <int R, bool INV, typename C> struct MixDFT {
     }
 };
 
-constexpr int kGenMaxRadixRows = 16, kGenMaxRadixZ = 32;
+constexpr int kGenMaxRadixRows = 16, kGenMaxRadixZ = 16;
 
 // Stages with caller-supplied ends: the first stage reads its inputs through
 // ld(row, col) (global memory, with the pass's prologue) and the last stage

@@ -349,7 +349,7 @@ bool zws_ok(int L, const void *S, const void *ntile, int nrows, int64_t ss, int6
 template <typename T>
 size_t Passes<T>::tile_tensor_elems(int L, int Py, int Kx)
 {
-    if (sizeof(T) != 4 || (L != 256 && L != 512)) return 0;
+    if (sizeof(T) != 4 || (L != 256 && L != 512 && (pow2_len(L) || !MixedPasses<T>::z_tiled(L)))) return 0;
     return (size_t)(Py / 2 + 1) * zws_ntx4(Kx) * 24 * (L / 2 + 1);  // [hy][ntx4][6][HZ][4]
 }
 
@@ -710,10 +710,10 @@ cudaError_t Passes<T>::zconv_pipe(C *S, int ncols, int width, int64_t ss, int64_
 template <typename T>
 cudaError_t Passes<T>::zconv(int L, C *S, int ncols, int width, int64_t ss, int64_t rs, int64_t cs,
                              int nrows, const T *nhat, int Py, int Kx, const C *tw, int twstride,
-                             cudaStream_t st, int variant)
+                             cudaStream_t st, int variant, const T *ntile)
 {
     if (ncols > 0 && !pow2_len(L))
-        return MixedPasses<T>::zconv(L, S, ncols, width, ss, rs, cs, nrows, nhat, Py, Kx, tw, twstride, st);
+        return MixedPasses<T>::zconv(L, S, ncols, width, ss, rs, cs, nrows, nhat, Py, Kx, tw, twstride, st, ntile);
     if (variant == 5 && ncols > 0 && 2 * nrows <= L) {
         cudaError_t e = cudaErrorNotSupported;
         switch (L) {

@@ -54,7 +54,10 @@ template <typename T> struct MixedPasses {
     static cudaError_t col(int L, bool inv, const C *in, C *out, int ncols, int width, int64_t iss, int64_t irs,
                            int nin, int64_t oss, int64_t ors, int nout, const C *tw, int twstride, cudaStream_t st);
     static cudaError_t zconv(int L, C *S, int ncols, int width, int64_t ss, int64_t rs, int64_t cs, int nrows,
-                             const T *nhat, int Py, int Kx, const C *tw, int twstride, cudaStream_t st);
+                             const T *nhat, int Py, int Kx, const C *tw, int twstride, cudaStream_t st,
+                             const T *ntile);
+    // whether the z pass of length L reads the tile-ordered tensor copy
+    static bool z_tiled(int L);
     static cudaError_t sp_zconv(int L, C *S, int ncols, int width, int64_t ss, int64_t rs, int64_t cs, int nrows,
                                 int nout, const T *that, int Py, int Kx, const C *tw, const C *phx, const C *phy,
                                 const C *phz, cudaStream_t st);
@@ -87,7 +90,7 @@ template <typename T> struct Passes {
     // fused z forward, spectral product, z inverse (in place)
     static cudaError_t zconv(int L, C *S, int ncols, int width, int64_t ss, int64_t rs, int64_t cs,
                              int nrows, const T *nhat, int Py, int Kx, const C *tw, int twstride,
-                             cudaStream_t st, int variant = 0);
+                             cudaStream_t st, int variant = 0, const T *ntile = nullptr);
     // persistent z pass streaming column tiles by TMA (FP32, L = 256 or 512, at
     // most L/2 input rows); ntile: the tile-ordered tensor copy (tile_tensor); tc:
     // columns per tile, 8 (one CTA per SM) or 4 (two CTAs per SM). With
