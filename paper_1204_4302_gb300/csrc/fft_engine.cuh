@@ -271,18 +271,21 @@ __device__ __forceinline__ T cell_weight(const T *wcell, int row, int rows_per_c
     return wcell ? __ldg(&wcell[(int64_t)(row % rows_per_comp) * rs + x]) : (T)1;
 }
 
-// Block sum of a per-thread double into partials[slot] (slot = the tile).
+// Block sum of a per-thread double into partials[slot] (slot = the tile). The
+// FP64 pipe is narrow on this GPU, so one warp adds the values (NT / 32 per
+// lane, then five shuffle levels) instead of every warp running its own levels.
 template <int NT>
 __device__ __forceinline__ void block_partial(double v, double *partials, int slot)
 {
-    __shared__ double red[NT / 32];
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __shared__ double red[NT];
+    red[threadIdx.x] = v;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0;
-        for (int w = 0; w < NT / 32; ++w) s += red[w];
-        partials[slot] = s;
+    if (threadIdx.x < 32) {
+        double s = red[threadIdx.x];
+#pragma unroll
+        for (int w = 1; w < NT / 32; ++w) s += red[threadIdx.x + 32 * w];
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+        if (threadIdx.x == 0) partials[slot] = s;
     }
 }
 
