@@ -371,7 +371,7 @@ __global__ void k_extract(const double2 *__restrict__ S, int comp, int Kx, int P
     block_max_to(local, imag_max);
 }
 
-constexpr int kFinalizeThreads = 256;
+constexpr int kFinalizeThreads = 128;
 
 // Compensated pair sum (s, c) + (s2, c2) -> (s, c): Neumaier's two-sum of the
 // leading parts, the error and both compensations in c.
@@ -392,36 +392,36 @@ __device__ __forceinline__ void warp_two_sum(double &s, double &c)
     }
 }
 
-// Sum of n FP64 partials times `factor` into *E. The CUDA cores' FP64 rate
-// per SM is low on this GPU, so the sum is spread over up to kFinalizeBlocks
-// CTAs and kept shallow: CTA b sums the contiguous chunk b (Neumaier-
-// compensated per thread, then warp shuffles and one shared-memory step over
-// the warps) into scratch[2b], scratch[2b + 1]; the CTA that finishes last (a
-// counter after the scratch) combines the CTA results the same way in its
-// first two warps, writes *E and resets the counter. The pairing is fixed, so
-// the result does not depend on which CTA finishes last.
+// Sum of n FP64 partials times `factor` into *E. A warp's FP64 instruction
+// holds the SM's narrow FP64 pipe for 16 cycles, so what bounds this kernel is
+// the number of compensated adds a CTA runs in all its warps: CTA b takes the
+// contiguous chunk b (one value per thread up to kFinalizeBlocks CTAs), leaves
+// the values in shared memory, and one warp adds them (four per lane, then
+// five shuffle levels) into scratch[2b], scratch[2b + 1]; the CTA that finishes
+// last (a counter after the scratch) combines the CTA results the same way, writes
+// *E and resets the counter. The pairing is fixed, so the result does not depend on
+// which CTA finishes last. With shuffle levels in all eight warps of 256 threads
+// it took 10 us for 500 partials.
 __global__ void __launch_bounds__(kFinalizeThreads) k_energy_finalize(const double *__restrict__ partials, int n,
                                                                       double factor, double *__restrict__ E,
                                                                       double *__restrict__ scratch)
 {
     constexpr int NW = kFinalizeThreads / 32;
-    __shared__ double ss[NW], sc[NW];
+    __shared__ double ss[kFinalizeThreads], sc[kFinalizeThreads];
     __shared__ bool s_last;
     const int nb = gridDim.x, chunk = (n + nb - 1) / nb;
     const int lo = blockIdx.x * chunk, hi = min(n, lo + chunk);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double s = 0.0, c = 0.0;
-    for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) two_sum_add(s, c, partials[i], 0.0);
-    warp_two_sum(s, c);
-    if (lane == 0) {
-        ss[warp] = s;
-        sc[warp] = c;
-    }
+    int i = lo + threadIdx.x;
+    double s = i < hi ? partials[i] : 0.0, c = 0.0;
+    for (i += blockDim.x; i < hi; i += blockDim.x) two_sum_add(s, c, partials[i], 0.0);
+    ss[threadIdx.x] = s;
+    sc[threadIdx.x] = c;
     __syncthreads();
     unsigned int *count = reinterpret_cast<unsigned int *>(scratch + 2 * kFinalizeBlocks);
     if (warp == 0) {
-        s = lane < NW ? ss[lane] : 0.0;
-        c = lane < NW ? sc[lane] : 0.0;
+#pragma unroll
+        for (int w = 1; w < NW; ++w) two_sum_add(s, c, ss[lane + 32 * w], sc[lane + 32 * w]);
         warp_two_sum(s, c);
         if (lane == 0) {
             scratch[2 * blockIdx.x] = s;
