@@ -477,9 +477,12 @@ demag_status demag_tune_padding(int nx, int ny, int nz, double dx, double dy, do
  *    setup, about the size of the spectrum), both one tile ahead; the
  *    length-512 transforms run as 2 x 16 x 16 with packed FP32x2 butterflies
  *    (z length 512, at most 256 input rows), 7 = as 6 with 4-column tiles and
- *    two CTAs per SM, 8 = variant 0 with an 8-point second stage (8 complex
- *    values per component and thread across the product, half the registers
- *    and shared memory) and two CTAs per SM (z lengths 32..128).
+ *    two CTAs per SM, 8 = an 8-point second stage (z lengths 32..128): FP64,
+ *    variant 0 with half the registers and shared memory and two CTAs per SM;
+ *    FP32, small tiles of 64 to 128 threads that read the tile-ordered tensor
+ *    copy, several CTAs per SM.
+ *    SP plans have one form per length, and 5 (lengths 32..256); FP32 SP plans of
+ *    z length 256 and 512 run persistent TMA-fed tiles whatever the variant.
  * y: 0 = two-stage column transform, 1 = swapped radix order (y lengths 32,
  *    128, 512), 2 = three-stage transform with more CTAs per SM (y lengths
  *    512 and 1024), 3 = as 2, with the forward pass by persistent CTAs that

@@ -316,13 +316,14 @@ struct FieldJob {
     double *E_dev;        // optional energy -(mu0/2) V sum input . H
 };
 
-// Field calls with the energy take its spectral sum in the persistent z pass
-// (FP32 plans of the tensor method whose z form is 6 or 7 at length 256 or
-// 512, spectral route on); the last pass then does not read M.
+// Field calls with the energy take its spectral sum in the z pass (FP32 plans
+// of the tensor method whose z form is 6 or 7 at length 256 or 512, or 8 at
+// lengths 32 to 128, spectral route on); the last pass then does not read M.
 bool energy_in_z(const demag_plan *p)
 {
     return p->method == DEMAG_METHOD_DM && p->prec == DEMAG_F32 && p->spectral_energy && p->ntile &&
-           (p->zvariant == 6 || p->zvariant == 7) && (p->Pz == 256 || p->Pz == 512);
+           (((p->zvariant == 6 || p->zvariant == 7) && (p->Pz == 256 || p->Pz == 512)) ||
+            (p->zvariant == 8 && (p->Pz == 32 || p->Pz == 64 || p->Pz == 128)));
 }
 
 template <typename T>
@@ -382,6 +383,11 @@ demag_status run_field(demag_plan *p, const FieldJob &job, cudaStream_t st)
             e = Passes<T>::zconv_ws_energy(Pz, S2, Kx, Py, Kxp, (int64_t)Py * Kxp, (int64_t)nz * Py * Kxp, nz,
                                            (const T *)(const void *)p->ntile, twz, p->partials, &nparts, st,
                                            p->zvariant == 7 ? 4 : 8);
+        if (e == cudaErrorNotSupported && f32 && p->ntile) {
+            nparts = p->npartials;
+            e = Passes<T>::zconv_t(Pz, S2, Kx, Py, Kxp, (int64_t)Py * Kxp, (int64_t)nz * Py * Kxp, nz,
+                                   (const T *)(const void *)p->ntile, twz, st, false, p->partials, &nparts);
+        }
         if (e == cudaErrorNotSupported)
             e = Passes<T>::zconv_energy(Pz, S2, Py * Kx, Kx, Kxp, (int64_t)Py * Kxp, (int64_t)nz * Py * Kxp, nz, nhat,
                                         Py, Kx, twz, 1, p->partials, &nparts, st);
@@ -409,6 +415,10 @@ demag_status run_field(demag_plan *p, const FieldJob &job, cudaStream_t st)
         e = Passes<T>::zconv_ws(Pz, S2, Kx, Py, Kxp, (int64_t)Py * Kxp, (int64_t)nz * Py * Kxp, nz,
                                 (const T *)(const void *)p->ntile, twz, st, p->zvariant == 7 ? 4 : 8,
                                 zenergy ? p->partials : nullptr, zenergy ? &zparts : nullptr);
+    else if (p->zvariant == 8 && f32 && p->ntile)
+        e = Passes<T>::zconv_t(Pz, S2, Kx, Py, Kxp, (int64_t)Py * Kxp, (int64_t)nz * Py * Kxp, nz,
+                               (const T *)(const void *)p->ntile, twz, st, true, zenergy ? p->partials : nullptr,
+                               zenergy ? &zparts : nullptr);
     if (!(e == cudaSuccess && zenergy)) zparts = 0;
     if (zparts > 0) {
         xo.Mref = nullptr;
@@ -435,7 +445,7 @@ demag_status run_field(demag_plan *p, const FieldJob &job, cudaStream_t st)
         nblocks = p->npartials;
         e = Passes<T>::x1_inv(S1, rows, xo, nblocks, st);
     } else {
-        nblocks = Passes<T>::x_blocks(Px / 2, rows);
+        nblocks = Passes<T>::x_blocks(Px / 2, rows, p->xvariant);
         e = Passes<T>::x_inv(Px / 2, S1, Kxp, rows, nx, xo, twx, st, p->xvariant);
     }
     if (e != cudaSuccess) return fail(DEMAG_ERR_CUDA, std::string("x inverse: ") + cudaGetErrorString(e));
@@ -502,7 +512,7 @@ demag_status run_field_sp(demag_plan *p, const FieldJob &job, cudaStream_t st)
     p->launches++;
     tm.mark();
     e = Passes<T>::sp_zconv(Pz, S2, Py * Kx, Kx, Kxp, (int64_t)Py * Kxp, (int64_t)nz * Py * Kxp, nz, nz + 1, that, Py,
-                            Kx, twz, phx, phy, phz, st, p->zvariant);
+                            Kx, twz, phx, phy, phz, st, p->zvariant, f32 ? (const T *)(const void *)p->ntile : nullptr);
     if (e != cudaSuccess) return fail(DEMAG_ERR_CUDA, std::string("SP z pass: ") + cudaGetErrorString(e));
     p->launches++;
     tm.mark();
@@ -692,7 +702,7 @@ std::string tune_key(const demag_plan *p)
     for (auto &c : name)
         if (c == ' ') c = '_';
     char buf[256];
-    snprintf(buf, sizeof buf, "v2|%s|%s|%dx%dx%d|%dx%dx%d%s", name.c_str(), p->prec == DEMAG_F32 ? "f32" : "f64", p->Px,
+    snprintf(buf, sizeof buf, "v3|%s|%s|%dx%dx%d|%dx%dx%d%s", name.c_str(), p->prec == DEMAG_F32 ? "f32" : "f64", p->Px,
              p->Py, p->Pz, p->nx, p->ny, p->nz, p->method == DEMAG_METHOD_SP ? "|sp" : "");
     return buf;
 }
@@ -887,8 +897,9 @@ size_t table_count(const demag_plan *p)
 // z length that kernel does not support keep none.
 cudaError_t build_ntile(demag_plan *p, cudaStream_t st)
 {
-    if (p->prec != DEMAG_F32 || p->method != DEMAG_METHOD_DM || !p->nhat32) return cudaSuccess;
-    const size_t n = Passes<float>::tile_tensor_elems(p->Pz, p->Py, p->Kx);
+    if (p->prec != DEMAG_F32 || !p->nhat32) return cudaSuccess;
+    const bool sp = p->method == DEMAG_METHOD_SP;
+    const size_t n = Passes<float>::tile_tensor_elems(p->Pz, p->Py, p->Kx, sp);
     if (n == 0) return cudaSuccess;
     if (!p->ntile) {
         cudaError_t e = dmalloc(&p->ntile, n * sizeof(float));
@@ -899,7 +910,7 @@ cudaError_t build_ntile(demag_plan *p, cudaStream_t st)
         p->ntile_bytes = n * sizeof(float);
         p->device_bytes += p->ntile_bytes;
     }
-    return Passes<float>::tile_tensor(p->Pz, p->nhat32, p->ntile, p->Py, p->Kx, st);
+    return Passes<float>::tile_tensor(p->Pz, p->nhat32, p->ntile, p->Py, p->Kx, st, sp);
 }
 
 // A plan that is only timed (padding autotuner): its tensor spectrum is
@@ -1116,6 +1127,7 @@ demag_status sp_setup(demag_plan *p, cudaStream_t st)
                                        (int64_t)Py * Kxp, Pz, p->tw64[2], 1, st));
         SETUP_CUDA(demag::sp_extract(St, c, Px, Py, Pz, Kxp, t64, p->nhat32, imag, st));
     }
+    SETUP_CUDA(build_ntile(p, st));
     unsigned long long bits = 0;
     SETUP_CUDA(cudaMemcpyAsync(&bits, imag, sizeof(bits), cudaMemcpyDeviceToHost, st));
     SETUP_CUDA(cudaStreamSynchronize(st));
@@ -1620,7 +1632,7 @@ demag_status demag_tune_padding(int nx, int ny, int nz, double dx, double dy, do
     for (auto &c : name)
         if (c == ' ') c = '_';
     char key[256];
-    snprintf(key, sizeof key, "pad1|%s|%s|%dx%dx%d", name.c_str(), prec == DEMAG_F32 ? "f32" : "f64", nx, ny, nz);
+    snprintf(key, sizeof key, "pad2|%s|%s|%dx%dx%d", name.c_str(), prec == DEMAG_F32 ? "f32" : "f64", nx, ny, nz);
     const std::string kbest = std::string(key) + "|best", kpow2 = std::string(key) + "|pow2";
     int c0, c1, c2, q0, q1, q2;
     double mb = 0, mp = 0;

@@ -31,6 +31,7 @@
 #include <vector>
 
 #include "fft2.cuh"
+#include "zt.cuh"
 #include "plan.h"
 
 namespace demag {
@@ -50,13 +51,11 @@ struct PassGeom {
 
 template <int L> constexpr size_t x_smem()
 {
-    if constexpr (L >= 64) return (size_t)XShape<float, L>::TR * XShape<float, L>::RS * 8;
-    else return (size_t)swsize(L * TileShape<float, L>::TC) * 8;
+    return (size_t)XShape<float, L>::TR * XShape<float, L>::RS * 8;
 }
 template <int L> constexpr int x_rows()
 {
-    if constexpr (L >= 64) return XShape<float, L>::TR;
-    else return TileShape<float, L>::TC;
+    return XShape<float, L>::TR;
 }
 
 bool x_geom(int L, int &rows_per_tile, size_t &sm)
@@ -85,24 +84,60 @@ bool y_geom(int L, int &cols_per_tile, size_t &sm)
     return false;
 }
 
-// z tiles of the batch kernels: the 8-point second stage (variant 8) for
-// lengths 32..128, the two-stage variant 0 otherwise.
-template <int L> constexpr int kBatchZV = (L >= 32 && L <= 128) ? 8 : 0;
+// z lengths 32..128 run the small-tile z pass (k_z_t's tile): one tile per CTA in
+// the pass-batched launches, one per thread group in the persistent kernel.
+template <int L> constexpr int kBatchZC = kZtCols<L>;
+template <int PASS, int L> constexpr bool kBatchZt = PASS == 2 && L >= 32 && L <= 128;
+template <int PASS, int L> constexpr int batch_threads()
+{
+    if constexpr (kBatchZt<PASS, L>) return ZtShape<L, kBatchZC<L>>::NT;
+    else return kThreads;
+}
+// Resident CTAs the launch bounds ask for: the row and column passes are bound by
+// the loads in flight (five CTAs of at most 48 registers; the x inverse pass keeps four).
+template <int PASS, int L> constexpr int batch_min_ctas()
+{
+    if constexpr (kBatchZt<PASS, L>) return 512 / batch_threads<PASS, L>();
+    else if constexpr ((PASS == 0 && L <= 256) || ((PASS == 1 || PASS == 3) && L <= 256)) return 5;
+    else if constexpr (PASS == 4 && L <= 256) return 4;
+    else return 1;
+}
+// Its tiles of one state (0: the state's z length runs another tile).
+int zt_batch_items(int L, int Py, int Kx)
+{
+    if (L < 32 || L > 128) return 0;
+    const int tc = L == 32 ? kBatchZC<32> : (L == 64 ? kBatchZC<64> : kBatchZC<128>);
+    return (Kx + tc - 1) / tc * Py;
+}
+// Tiles per item of the persistent kernel.
+int zt_batch_groups(int L)
+{
+    return kThreads / (L == 32 ? ZtShape<32, kBatchZC<32>>::NT : L == 64 ? ZtShape<64, kBatchZC<64>>::NT : ZtShape<128, kBatchZC<128>>::NT);
+}
+size_t zt_batch_smem(int L)
+{
+    return L == 32 ? ZtShape<32, kBatchZC<32>>::SMEM : L == 64 ? ZtShape<64, kBatchZC<64>>::SMEM : ZtShape<128, kBatchZC<128>>::SMEM;
+}
 
 template <int L> constexpr size_t z_smem()
 {
-    using Sh = ZShape<float, L, kBatchZV<L>>;
-    return 3 * swsize(L * Sh::TC) * 8 + (size_t)(L / 2 + 1) * 6 * Sh::TC * 4;
+    if constexpr (L <= 128) {
+        using Sh = ZtShape<L, kBatchZC<L>>;
+        return kThreads / Sh::NT * Sh::SMEM;
+    } else {
+        using Sh = ZShape<float, L, 0>;
+        return 3 * swsize(L * Sh::TC) * 8 + (size_t)(L / 2 + 1) * 6 * Sh::TC * 4;
+    }
 }
 
 bool z_geom(int L, int &cols_per_tile, size_t &sm)
 {
     switch (L) {
     case 4: case 8: case 16: cols_per_tile = kThreads; sm = 0; return true;
-    case 32: cols_per_tile = ZShape<float, 32, kBatchZV<32>>::TC; sm = z_smem<32>(); return true;
-    case 64: cols_per_tile = ZShape<float, 64, kBatchZV<64>>::TC; sm = z_smem<64>(); return true;
-    case 128: cols_per_tile = ZShape<float, 128, kBatchZV<128>>::TC; sm = z_smem<128>(); return true;
-    case 256: cols_per_tile = ZShape<float, 256, kBatchZV<256>>::TC; sm = z_smem<256>(); return true;
+    case 32: cols_per_tile = 0; sm = z_smem<32>(); return true;
+    case 64: cols_per_tile = 0; sm = z_smem<64>(); return true;
+    case 128: cols_per_tile = 0; sm = z_smem<128>(); return true;
+    case 256: cols_per_tile = ZShape<float, 256, 0>::TC; sm = z_smem<256>(); return true;
     }
     return false;
 }
@@ -124,17 +159,17 @@ bool pass_geom(const demag_plan *p, PassGeom &g)
         g.smem[3] = g.smem[1];
     }
     if (!z_geom(p->Pz, per, g.smem[2])) return false;
-    g.tiles[2] = (p->Py * p->Kx + per - 1) / per;
+    const int zt = zt_batch_items(p->Pz, p->Py, p->Kx), groups = zt_batch_groups(p->Pz);
+    g.tiles[2] = zt ? (zt + groups - 1) / groups : (p->Py * p->Kx + per - 1) / per;
     g.tiles[5] = 1;
     g.smem[5] = 0;
     return true;
 }
 
 // --------------------------------------------------------------- device side
-__device__ void energy_tile(const BatchState &st)
+__device__ void energy_tile(const BatchState &st, int n, double factor)
 {
     __shared__ double ss[kThreads], sc[kThreads];
-    const int n = st.ntiles[4];
     double s = 0.0, c = 0.0;
     for (int i = threadIdx.x; i < n; i += kThreads) {
         const double v = __ldcg(&st.partials[i]);
@@ -155,7 +190,19 @@ __device__ void energy_tile(const BatchState &st)
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0 && st.E) *st.E = st.efactor * (ss[0] + sc[0]);
+    if (threadIdx.x == 0 && st.E) *st.E = factor * (ss[0] + sc[0]);
+}
+
+// One item of the persistent kernel at z lengths 32..128: a tile per thread group.
+template <int L>
+__device__ __forceinline__ void zt_group(const BatchState &st, int item, unsigned char *sm)
+{
+    using Sh = ZtShape<L, kBatchZC<L>>;
+    const int tile = item * (kThreads / Sh::NT) + (int)threadIdx.x / Sh::NT;
+    if (tile < st.nez)
+        zt_tile<L, kBatchZC<L>, ZT_BOTH, true>(st.S2, st.Kx, st.Py, st.Kxp, (int64_t)st.Py * st.Kxp,
+                                               (int64_t)st.nz * st.Py * st.Kxp, st.nz, st.ntile, st.tw[2],
+                                               (st.Kx + kBatchZC<L> - 1) / kBatchZC<L>, tile, sm, st.partials);
 }
 
 template <int PASS>
@@ -169,8 +216,8 @@ __device__ __forceinline__ void run_item_t(const BatchState &st, int tile, unsig
         XIn<float> a;
         a.in = st.M; a.in_rs = nx; a.wcell = nullptr; a.wscalar = 1.f; a.rows_per_comp = nz * ny;
         switch (Px / 2) {
-        case 16: k_x_fwd_tile<float, 16, false>(a, rows, nx, st.S1, Kxp, st.tw[0], tile, sm); break;
-        case 32: k_x_fwd_tile<float, 32, false>(a, rows, nx, st.S1, Kxp, st.tw[0], tile, sm); break;
+        case 16: k_x_fwd2_tile<float, 16, true, false>(a, rows, nx, st.S1, Kxp, st.tw[0], tile, sm); break;
+        case 32: k_x_fwd2_tile<float, 32, true, false>(a, rows, nx, st.S1, Kxp, st.tw[0], tile, sm); break;
         case 64: k_x_fwd2_tile<float, 64, true, false>(a, rows, nx, st.S1, Kxp, st.tw[0], tile, sm); break;
         case 128: k_x_fwd2_tile<float, 128, true, false>(a, rows, nx, st.S1, Kxp, st.tw[0], tile, sm); break;
         case 256: k_x_fwd2_tile<float, 256, true, false>(a, rows, nx, st.S1, Kxp, st.tw[0], tile, sm); break;
@@ -215,20 +262,21 @@ __device__ __forceinline__ void run_item_t(const BatchState &st, int tile, unsig
         case 4: k_z_conv1_tile<float, 4, true>(st.S2, ncols, Kx, ss, rs, cs, nz, st.nhat, Py, Kx, tile, sm); break;
         case 8: k_z_conv1_tile<float, 8, true>(st.S2, ncols, Kx, ss, rs, cs, nz, st.nhat, Py, Kx, tile, sm); break;
         case 16: k_z_conv1_tile<float, 16, true>(st.S2, ncols, Kx, ss, rs, cs, nz, st.nhat, Py, Kx, tile, sm); break;
-        case 32: k_z_conv2_tile<float, 32, kBatchZV<32>, true>(st.S2, ncols, Kx, ss, rs, cs, nz, st.nhat, Py, Kx, st.tw[2], 1, tile, sm); break;
-        case 64: k_z_conv2_tile<float, 64, kBatchZV<64>, true>(st.S2, ncols, Kx, ss, rs, cs, nz, st.nhat, Py, Kx, st.tw[2], 1, tile, sm); break;
-        case 128: k_z_conv2_tile<float, 128, kBatchZV<128>, true>(st.S2, ncols, Kx, ss, rs, cs, nz, st.nhat, Py, Kx, st.tw[2], 1, tile, sm); break;
-        case 256: k_z_conv2_tile<float, 256, kBatchZV<256>, true>(st.S2, ncols, Kx, ss, rs, cs, nz, st.nhat, Py, Kx, st.tw[2], 1, tile, sm); break;
+        case 32: zt_group<32>(st, tile, sm); break;
+        case 64: zt_group<64>(st, tile, sm); break;
+        case 128: zt_group<128>(st, tile, sm); break;
+        case 256: k_z_conv2_tile<float, 256, 0, true>(st.S2, ncols, Kx, ss, rs, cs, nz, st.nhat, Py, Kx, st.tw[2], 1, tile, sm); break;
         }
         break;
     }
     case 4: {
         XOut<float> o;
         o.out = st.H; o.out_rs = nx; o.scale = 1.f / ((float)Px * Py * Pz); o.oscale = 1.f; o.wcell = nullptr;
-        o.gdev = nullptr; o.Mref = st.M; o.mscale = 1.f; o.partials = st.partials; o.rows_per_comp = nz * ny;
+        o.gdev = nullptr; o.Mref = st.nez ? nullptr : st.M; o.mscale = 1.f; o.partials = st.nez ? nullptr : st.partials;
+        o.rows_per_comp = nz * ny;
         switch (Px / 2) {
-        case 16: k_x_inv_tile<float, 16, true>(st.S1, Kxp, rows, nx, o, st.tw[0], tile, sm); break;
-        case 32: k_x_inv_tile<float, 32, true>(st.S1, Kxp, rows, nx, o, st.tw[0], tile, sm); break;
+        case 16: k_x_inv2_tile<float, 16, true>(st.S1, Kxp, rows, nx, o, st.tw[0], tile, sm); break;
+        case 32: k_x_inv2_tile<float, 32, true>(st.S1, Kxp, rows, nx, o, st.tw[0], tile, sm); break;
         case 64: k_x_inv2_tile<float, 64, true>(st.S1, Kxp, rows, nx, o, st.tw[0], tile, sm); break;
         case 128: k_x_inv2_tile<float, 128, true>(st.S1, Kxp, rows, nx, o, st.tw[0], tile, sm); break;
         case 256: k_x_inv2_tile<float, 256, true>(st.S1, Kxp, rows, nx, o, st.tw[0], tile, sm); break;
@@ -236,8 +284,9 @@ __device__ __forceinline__ void run_item_t(const BatchState &st, int tile, unsig
         }
         break;
     }
-    case 5:
-        energy_tile(st);
+    case 5:  // the z pass's sums where it takes them, else the x inverse pass's
+        if (st.nez) energy_tile(st, st.nez, st.ezfactor);
+        else energy_tile(st, st.ntiles[4], st.efactor);
         break;
     }
 }
@@ -265,8 +314,7 @@ __device__ __forceinline__ void run_item_L(const BatchState &st, int tile, unsig
     if constexpr (PASS == 0) {
         XIn<float> a;
         a.in = st.M; a.in_rs = nx; a.wcell = nullptr; a.wscalar = 1.f; a.rows_per_comp = nz * ny;
-        if constexpr (L <= 32) k_x_fwd_tile<float, L, false>(a, rows, nx, st.S1, Kxp, st.tw[0], tile, sm);
-        else k_x_fwd2_tile<float, L, true, false>(a, rows, nx, st.S1, Kxp, st.tw[0], tile, sm);
+        k_x_fwd2_tile<float, L, true, false>(a, rows, nx, st.S1, Kxp, st.tw[0], tile, sm);
     } else if constexpr (PASS == 1 || PASS == 3) {
         constexpr bool inv = PASS == 3;
         const float2 *in = inv ? st.S2 : st.S1;
@@ -287,16 +335,20 @@ __device__ __forceinline__ void run_item_L(const BatchState &st, int tile, unsig
         const int ncols = Py * Kx;
         const int64_t ss = Kxp, rs = (int64_t)Py * Kxp, cs = (int64_t)nz * Py * Kxp;
         if constexpr (L <= 16) k_z_conv1_tile<float, L, true>(st.S2, ncols, Kx, ss, rs, cs, nz, st.nhat, Py, Kx, tile, sm);
-        else k_z_conv2_tile<float, L, kBatchZV<L>, true>(st.S2, ncols, Kx, ss, rs, cs, nz, st.nhat, Py, Kx, st.tw[2], 1,
+        else if constexpr (L <= 128)
+            zt_tile<L, kBatchZC<L>, ZT_BOTH>(st.S2, Kx, Py, ss, rs, cs, nz, st.ntile, st.tw[2],
+                                              (Kx + kBatchZC<L> - 1) / kBatchZC<L>, tile, sm, st.partials);
+        else k_z_conv2_tile<float, L, 0, true>(st.S2, ncols, Kx, ss, rs, cs, nz, st.nhat, Py, Kx, st.tw[2], 1,
                                                         tile, sm);
     } else if constexpr (PASS == 4) {
         XOut<float> o;
         o.out = st.H; o.out_rs = nx; o.scale = 1.f / ((float)Px * Py * Pz); o.oscale = 1.f; o.wcell = nullptr;
-        o.gdev = nullptr; o.Mref = st.M; o.mscale = 1.f; o.partials = st.partials; o.rows_per_comp = nz * ny;
-        if constexpr (L <= 32) k_x_inv_tile<float, L, true>(st.S1, Kxp, rows, nx, o, st.tw[0], tile, sm);
-        else k_x_inv2_tile<float, L, true>(st.S1, Kxp, rows, nx, o, st.tw[0], tile, sm);
+        o.gdev = nullptr; o.Mref = st.nez ? nullptr : st.M; o.mscale = 1.f; o.partials = st.nez ? nullptr : st.partials;
+        o.rows_per_comp = nz * ny;
+        k_x_inv2_tile<float, L, true>(st.S1, Kxp, rows, nx, o, st.tw[0], tile, sm);
     } else {
-        energy_tile(st);
+        if (st.nez) energy_tile(st, st.nez, st.ezfactor);
+        else energy_tile(st, st.ntiles[4], st.efactor);
     }
 }
 
@@ -306,7 +358,7 @@ __device__ __forceinline__ void run_item_L(const BatchState &st, int tile, unsig
 // its m states gstate). The launches follow one another on the stream, so no
 // dependency waits are needed, and each launch carries one tile function.
 template <int PASS, int L>
-__global__ void __launch_bounds__(kThreads) k_batch_pass(BatchDesc d, const int *__restrict__ gstate,
+__global__ void __launch_bounds__(batch_threads<PASS, L>(), batch_min_ctas<PASS, L>()) k_batch_pass(BatchDesc d, const int *__restrict__ gstate,
                                                          const int *__restrict__ gstart, int m)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -494,7 +546,7 @@ demag_status build_persistent(demag_batch *b)
         }
         for (int k = 0; k < demag::kPasses; ++k)
             if (geo[i].tiles[k] > 0 && geo[i].smem[k] > smem) smem = geo[i].smem[k];
-        npart += geo[i].tiles[4];
+        npart += (size_t)std::max(geo[i].tiles[4], demag::zt_batch_items(b->plans[i]->Pz, b->plans[i]->Py, b->plans[i]->Kx));
     }
     if (smem > 227 * 1024) {
         b->why_not_persistent = "shared memory beyond one CTA";
@@ -512,9 +564,12 @@ demag_status build_persistent(demag_batch *b)
         s.S1 = (float2 *)p->S1;
         s.S2 = (float2 *)p->S2;
         s.nhat = p->nhat32;
+        s.ntile = p->ntile;
         for (int a = 0; a < 3; ++a) s.tw[a] = p->tw32[a];
         s.partials = b->dpartials + poff;
-        poff += geo[i].tiles[4];
+        s.nez = demag::zt_batch_items(p->Pz, p->Py, p->Kx);
+        s.ezfactor = 0.5 * demag::kMu0 * p->dx * p->dy * p->dz / ((double)p->Px * p->Py * p->Pz);
+        poff += (size_t)std::max(geo[i].tiles[4], s.nez);
         s.E = b->dE + i;
         s.nx = p->nx; s.ny = p->ny; s.nz = p->nz;
         s.Px = p->Px; s.Py = p->Py; s.Pz = p->Pz; s.Kx = p->Kx; s.Kxp = p->Kxp;
@@ -561,9 +616,11 @@ demag_status build_persistent(demag_batch *b)
                     const demag_plan_t pl = b->plans[i];
                     const int Li = (k == 0 || k == 4) ? pl->Px / 2 : (k == 1 || k == 3) ? pl->Py : (k == 2 ? pl->Pz : 0);
                     if (Li != L) continue;
+                    const bool zt = k == 2 && L >= 32 && L <= 128;
+                    const size_t sm = zt ? demag::zt_batch_smem(L) : geo[i].smem[k];
                     st.push_back(i);
-                    pre.push_back(pre.back() + geo[i].tiles[k]);
-                    if (geo[i].smem[k] > g.smem) g.smem = geo[i].smem[k];
+                    pre.push_back(pre.back() + (zt ? demag::zt_batch_items(L, pl->Py, pl->Kx) : geo[i].tiles[k]));
+                    if (sm > g.smem) g.smem = sm;
                 }
                 g.m = (int)st.size();
                 g.items = pre.back();
@@ -670,7 +727,7 @@ cudaError_t group_launch(demag_batch *b, const BatchDesc &d, const demag_batch::
         if (e != cudaSuccess) return e;
         done_for = b->device;
     }
-    demag::k_batch_pass<PASS, L><<<g.items, demag::kThreads, g.smem, st>>>(d, b->dgroups + g.off,
+    demag::k_batch_pass<PASS, L><<<g.items, demag::batch_threads<PASS, L>(), g.smem, st>>>(d, b->dgroups + g.off,
                                                                            b->dgroups + g.off + g.m, g.m);
     return cudaGetLastError();
 }
@@ -1056,9 +1113,12 @@ demag_status demag_batch_autotune(demag_batch_t b, int use_cache, double *ms_per
     b->timing = timing;
     release();
     if (rs != DEMAG_OK) return rs;
-    int best = 1;
-    for (int m = 0; m < 3; ++m)
-        if (t[m] < t[best]) best = m;
+    // the branch graph is rebuilt whenever a call brings other buffers (6 ms for 64
+    // states against a call of 1.4 ms), the other modes upload a table: it is taken
+    // where it is faster by a tenth
+    int best = b->persistent_ok ? 2 : 1;
+    if (t[0] < t[best]) best = 0;
+    if (t[1] < 0.9 * t[best]) best = 1;
     b->mode = best;
     b->tuned_ms[0] = t[0]; b->tuned_ms[1] = t[1]; b->tuned_ms[2] = t[2];
     if (ms_persistent) *ms_persistent = b->persistent_ok ? t[0] : -1.0;

@@ -857,15 +857,17 @@ namespace demag {
 // R1 - j2 at r' = R2 - 1 - r (thread 0 holds its own partners), exchanged by
 // warp shuffles.
 template <int L> struct XRadix;
+template <> struct XRadix<16> { static constexpr int R1 = 4, R2 = 4; };
+template <> struct XRadix<32> { static constexpr int R1 = 8, R2 = 4; };
 template <> struct XRadix<64> { static constexpr int R1 = 8, R2 = 8; };
 template <> struct XRadix<128> { static constexpr int R1 = 16, R2 = 8; };
 template <> struct XRadix<256> { static constexpr int R1 = 16, R2 = 16; };
 template <> struct XRadix<512> { static constexpr int R1 = 32, R2 = 16; };
 
-template <typename T, int L> struct XShape {
+template <typename T, int L, int NTX = Tile2<T>::NT> struct XShape {
     static constexpr int R1 = XRadix<L>::R1, R2 = XRadix<L>::R2;
     static_assert(R1 <= 32 && 32 % R1 == 0, "the exchange indexing assumes R1 divides 32");
-    static constexpr int NT = Tile2<T>::NT;
+    static constexpr int NT = NTX;
     static constexpr int TR = NT / (R1 > R2 ? R1 : R2);  // rows per CTA
     static constexpr int RS = swsize(L);                 // padded row in shared memory
 };
@@ -895,12 +897,12 @@ __device__ __forceinline__ C shfl_c(C v, int lane)
 // Real-to-complex along x (see k_x_fwd for the packing), two stages.
 // PIN: the row has at most L reals (the zero-padded field), so the upper half
 // of the packed sequence is zero; otherwise all 2L reals are read (setup).
-template <typename T, int L, bool PIN, bool CG>
+template <typename T, int L, bool PIN, bool CG, int NTX = Tile2<T>::NT>
 __device__ __forceinline__ void k_x_fwd2_tile(XIn<T> a, int nrows, int nvalid, typename Cplx<T>::type *__restrict__ out, int64_t out_rs,
          const typename Cplx<T>::type *__restrict__ twx, int tile, unsigned char *smraw)
 {
     using C = typename Cplx<T>::type;
-    using S = XShape<T, L>;
+    using S = XShape<T, L, NTX>;
     constexpr int R1 = S::R1, R2 = S::R2, TR = S::TR, RS = S::RS;
     C *sm = reinterpret_cast<C *>(smraw);
     const int row0 = tile * TR;
@@ -910,30 +912,39 @@ __device__ __forceinline__ void k_x_fwd2_tile(XIn<T> a, int nrows, int nvalid, t
         C u[R1];
 #pragma unroll
         for (int r = 0; r < R1; ++r) u[r] = cmk<C>(0, 0);
-        if (row < nrows) {
-            const T *p = a.in + (int64_t)row * a.in_rs;
-            const T ws = a.wscalar;
-            if ((a.in_rs & 1) == 0 && !a.wcell) {
-                // even rows: pairs are aligned, one vector load per complex value
+        // all loads first, independent and predicated, then the scaling
+        constexpr int H = PIN ? R1 / 2 : R1;
+        const T *p = a.in + (int64_t)row * a.in_rs;
+        const T ws = a.wscalar;
+        const int left = row < nrows ? nvalid : 0;
+        if (((a.in_rs | nvalid) & 1) == 0) {
+            // even rows: pairs are aligned, one vector load per complex value
 #pragma unroll
-                for (int r = 0; r < (PIN ? R1 / 2 : R1); ++r) {
-                    const int x0 = 2 * (j1 + r * R2);
-                    if (x0 + 1 < nvalid) {
-                        const C q = *reinterpret_cast<const C *>(p + x0);
-                        u[r] = cmk<C>(q.x * ws, q.y * ws);
-                    } else if (x0 < nvalid) {
-                        u[r].x = p[x0] * ws;
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int r = 0; r < (PIN ? R1 / 2 : R1); ++r) {
-                    const int x0 = 2 * (j1 + r * R2);
-                    if (x0 < nvalid) u[r].x = p[x0] * ws * cell_weight(a.wcell, row, a.rows_per_comp, a.in_rs, x0);
-                    if (x0 + 1 < nvalid)
-                        u[r].y = p[x0 + 1] * ws * cell_weight(a.wcell, row, a.rows_per_comp, a.in_rs, x0 + 1);
-                }
+            for (int r = 0; r < H; ++r) {
+                const int x0 = 2 * (j1 + r * R2);
+                if (x0 < left) u[r] = *reinterpret_cast<const C *>(p + x0);
             }
+        } else {
+#pragma unroll
+            for (int r = 0; r < H; ++r) {
+                const int x0 = 2 * (j1 + r * R2);
+                if (x0 < left) u[r].x = p[x0];
+                if (x0 + 1 < left) u[r].y = p[x0 + 1];
+            }
+        }
+        if (a.wcell) {
+            const T *w = a.wcell + (int64_t)(row % a.rows_per_comp) * a.in_rs;
+#pragma unroll
+            for (int r = 0; r < H; ++r) {
+                const int x0 = 2 * (j1 + r * R2);
+                T w0 = 0, w1 = 0;
+                if (x0 < left) w0 = __ldg(&w[x0]);
+                if (x0 + 1 < left) w1 = __ldg(&w[x0 + 1]);
+                u[r] = cmk<C>(u[r].x * ws * w0, u[r].y * ws * w1);
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < H; ++r) u[r] = cscale_rn(u[r], ws);
         }
         if constexpr (PIN) RegDFTHalfIn<R1, false, C>::run(u);
         else RegDFT<R1, false, C>::run(u);
@@ -971,13 +982,13 @@ __device__ __forceinline__ void k_x_fwd2_tile(XIn<T> a, int nrows, int nvalid, t
     }
 }
 
-template <typename T, int L, bool PIN>
-__global__ void __launch_bounds__(Tile2<T>::NT)
+template <typename T, int L, bool PIN, int NTX = Tile2<T>::NT>
+__global__ void __launch_bounds__(NTX)
 k_x_fwd2(XIn<T> a, int nrows, int nvalid, typename Cplx<T>::type *__restrict__ out, int64_t out_rs,
          const typename Cplx<T>::type *__restrict__ twx)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
-    k_x_fwd2_tile<T, L, PIN, false>(a, nrows, nvalid, out, out_rs, twx, blockIdx.x, smraw);
+    k_x_fwd2_tile<T, L, PIN, false, NTX>(a, nrows, nvalid, out, out_rs, twx, blockIdx.x, smraw);
 }
 
 // Complex-to-real along x (see k_x_inv), two stages, XOut epilogue. MP: the
@@ -1013,12 +1024,12 @@ __device__ __forceinline__ void x_out_pair(const XOut<T> &o, int row, int x, T h
     }
 }
 
-template <typename T, int L, bool CG, bool P1 = false, bool MP = false>
+template <typename T, int L, bool CG, bool P1 = false, bool MP = false, int NTX = Tile2<T>::NT>
 __device__ __forceinline__ void k_x_inv2_tile(const typename Cplx<T>::type *__restrict__ in, int64_t in_rs, int nrows, int nvalid, XOut<T> o,
          const typename Cplx<T>::type *__restrict__ twx, int tile, unsigned char *smraw)
 {
     using C = typename Cplx<T>::type;
-    using S = XShape<T, L>;
+    using S = XShape<T, L, NTX>;
     constexpr int R1 = S::R1, R2 = S::R2, NT = S::NT, TR = S::TR, RS = S::RS;
     C *sm = reinterpret_cast<C *>(smraw);
     T *smM = reinterpret_cast<T *>(sm + TR * RS);  // MP: [TR][L] reference rows
@@ -1062,6 +1073,19 @@ __device__ __forceinline__ void k_x_inv2_tile(const typename Cplx<T>::type *__re
     if (threadIdx.x < TR * R1) {
         const int rr = threadIdx.x / R1, j2 = threadIdx.x % R1, row = row0 + rr;
         const C *s = sm + rr * RS;
+        // the energy's M of a plain field's even rows, loaded ahead of the transform
+        constexpr int HO = P1 ? R2 / 2 + 1 : R2 / 2;
+        const bool ahead = !MP && o.partials && !o.wcell && ((o.out_rs | nvalid) & 1) == 0;
+        C m[HO];
+        if constexpr (!MP) {
+            const T *mp = o.Mref + (int64_t)row * o.out_rs;
+#pragma unroll
+            for (int r = 0; r < HO; ++r) {
+                m[r] = cmk<C>(0, 0);
+                if (ahead && row < nrows && 2 * (j2 + r * R1) < nvalid)
+                    m[r] = *reinterpret_cast<const C *>(mp + 2 * (j2 + r * R1));
+            }
+        }
         C v[R2];
 #pragma unroll
         for (int r = 0; r < R2; ++r) v[r] = s[xex<R1>(r, j2)];
@@ -1072,8 +1096,18 @@ __device__ __forceinline__ void k_x_inv2_tile(const typename Cplx<T>::type *__re
         if (row < nrows) {
             const T g = o.gdev ? (T)(*o.gdev) : (T)1;
             const T oscale = o.oscale * g;
+            if (ahead) {
+                T *op = o.out + (int64_t)row * o.out_rs;
 #pragma unroll
-            for (int r = 0; r < (P1 ? R2 / 2 + 1 : R2 / 2); ++r) {  // z[n], n = j2 + r R1 (< L/2 unless P1)
+                for (int r = 0; r < HO; ++r) {  // m is zero beyond the row
+                    const C hv = cmk<C>(v[r].x * o.scale, v[r].y * o.scale);
+                    if (o.out && 2 * (j2 + r * R1) < nvalid)
+                        *reinterpret_cast<C *>(op + 2 * (j2 + r * R1)) = cmk<C>(hv.x * oscale, hv.y * oscale);
+                    acc += o.mscale * (m[r].x * hv.x + m[r].y * hv.y);
+                }
+            } else
+#pragma unroll
+            for (int r = 0; r < HO; ++r) {  // z[n], n = j2 + r R1 (< L/2 unless P1)
                 const int n = j2 + r * R1;
                 x_out_pair<T>(o, row, 2 * n, v[r].x * o.scale, v[r].y * o.scale, oscale, nvalid,
                               MP ? smM + rr * L : nullptr, acc);
@@ -1085,13 +1119,13 @@ __device__ __forceinline__ void k_x_inv2_tile(const typename Cplx<T>::type *__re
 
 // P1: one more output pair per row (x = L, L + 1, ...: rows of nx + 1 >= L
 // values, the node potential of the scalar-potential method).
-template <typename T, int L, bool P1 = false, bool MP = false>
-__global__ void __launch_bounds__(Tile2<T>::NT, (L >= 512 ? Occ<T, 2 * L>::MIN_CTAS : Occ<T, L>::MIN_CTAS))
+template <typename T, int L, bool P1 = false, bool MP = false, int NTX = Tile2<T>::NT>
+__global__ void __launch_bounds__(NTX, NTX < Tile2<T>::NT ? 8 : (L >= 512 ? Occ<T, 2 * L>::MIN_CTAS : Occ<T, L>::MIN_CTAS))
 k_x_inv2(const typename Cplx<T>::type *__restrict__ in, int64_t in_rs, int nrows, int nvalid, XOut<T> o,
          const typename Cplx<T>::type *__restrict__ twx)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
-    k_x_inv2_tile<T, L, false, P1, MP>(in, in_rs, nrows, nvalid, o, twx, blockIdx.x, smraw);
+    k_x_inv2_tile<T, L, false, P1, MP, NTX>(in, in_rs, nrows, nvalid, o, twx, blockIdx.x, smraw);
 }
 
 }  // namespace demag

@@ -11,7 +11,9 @@
 #include "launch_util.cuh"
 #include "plan.h"
 #include "sp.cuh"
+#include "spws.cuh"
 #include "xpipe.cuh"
+#include "zt.cuh"
 #include "zws.cuh"
 
 namespace demag {
@@ -43,9 +45,6 @@ __global__ void __launch_bounds__(256) k_x1_inv(const typename Cplx<T>::type *__
 }
 
 }  // namespace
-
-#define DEMAG_FOR_EACH_L(M) \
-    M(1) M(2) M(4) M(8) M(16) M(32) M(64) M(128) M(256) M(512) M(1024)
 
 namespace {
 // Resident CTAs per SM of a kernel at a given dynamic shared-memory size
@@ -347,21 +346,43 @@ bool zws_ok(int L, const void *S, const void *ntile, int nrows, int64_t ss, int6
 }  // namespace
 
 template <typename T>
-size_t Passes<T>::tile_tensor_elems(int L, int Py, int Kx)
+size_t Passes<T>::tile_tensor_elems(int L, int Py, int Kx, bool sp)
 {
-    if (sizeof(T) != 4 || (L != 256 && L != 512 && (pow2_len(L) || !MixedPasses<T>::z_tiled(L)))) return 0;
+    if (sp)  // the persistent SP z pass
+        return sizeof(T) == 4 && (L == 256 || L == 512) ? (size_t)(Py / 2 + 1) * zws_ntx4(Kx) * 12 * (L / 2 + 1) : 0;
+    if (sizeof(T) != 4 || (pow2_len(L) ? L < 32 || L > 512 : !MixedPasses<T>::z_tiled(L))) return 0;
     return (size_t)(Py / 2 + 1) * zws_ntx4(Kx) * 24 * (L / 2 + 1);  // [hy][ntx4][6][HZ][4]
 }
 
 template <typename T>
-cudaError_t Passes<T>::tile_tensor(int L, const T *nhat, T *ntile, int Py, int Kx, cudaStream_t st)
+cudaError_t Passes<T>::tile_tensor(int L, const T *nhat, T *ntile, int Py, int Kx, cudaStream_t st, bool sp)
 {
-    const size_t n = tile_tensor_elems(L, Py, Kx);
+    const size_t n = tile_tensor_elems(L, Py, Kx, sp);
     if (n == 0) return cudaErrorNotSupported;
     const int grid = (int)std::min<size_t>((n + 255) / 256, (size_t)sm_count() * 16);
-    k_tile_tensor<T><<<grid, 256, 0, st>>>(nhat, ntile, Kx, Py / 2 + 1, L / 2 + 1, zws_ntx4(Kx));
+    if (sp) k_tile_tensor<T, 3><<<grid, 256, 0, st>>>(nhat, ntile, Kx, Py / 2 + 1, L / 2 + 1, zws_ntx4(Kx));
+    else k_tile_tensor<T, 6><<<grid, 256, 0, st>>>(nhat, ntile, Kx, Py / 2 + 1, L / 2 + 1, zws_ntx4(Kx));
     return cudaGetLastError();
 }
+
+namespace {
+template <int L>
+cudaError_t spws_launch(float2 *S, int Kx, int Py, int64_t ss, int64_t rs, int64_t cs, int nrows, int nout, const float *ttile,
+                        const float2 *tw, const float2 *phx, const float2 *phy, const float2 *phz, cudaStream_t st)
+{
+    using Sh = SpwsShape<L>;
+    CUtensorMap map;
+    if (!zws_input_map<L, Sh::TC>(&map, S, Kx, Py, nrows, ss, rs, cs)) return cudaErrorNotSupported;
+    const size_t sm = spws_smem_bytes<L>(nrows);
+    cudaError_t e = allow_smem<k_sp_ws<L>>(sm);
+    if (e != cudaSuccess) return e;
+    const int ntx = (Kx + Sh::TC - 1) / Sh::TC, ntiles = ntx * Py;
+    const int cap = sm_count() * resident_ctas<k_sp_ws<L>>(Sh::NT, sm);
+    k_sp_ws<L><<<ntiles < cap ? ntiles : cap, Sh::NT, sm, st>>>(map, S, Kx, Py, ss, rs, nrows, nout, ttile, tw, phx, phy, phz,
+                                                               ntx, ntiles);
+    return cudaGetLastError();
+}
+}  // namespace
 
 template <typename T>
 cudaError_t Passes<T>::zconv_ws(int L, C *S, int Kx, int Py, int64_t ss, int64_t rs, int64_t cs, int nrows,
@@ -403,8 +424,53 @@ cudaError_t Passes<T>::zconv_ws_energy(int L, C *S, int Kx, int Py, int64_t ss, 
     }
 }
 
-// Spectral-energy z pass: the 8-point second stage (variant 8) for lengths
-// 32..128, as in the field pipeline's fastest form there.
+// Columns per tile of the small-tile z pass (see ZtShape).
+static int zt_cols(int L, int Py, int Kx)
+{
+    const int tc = L == 32 ? kZtCols<32> : L == 64 ? kZtCols<64> : kZtCols<128>;
+    return (Kx + tc - 1) / tc * Py < 2 * sm_count() ? 8 : tc;
+}
+
+template <typename T>
+cudaError_t Passes<T>::zconv_t(int L, C *S, int Kx, int Py, int64_t ss, int64_t rs, int64_t cs, int nrows, const T *ntile,
+                               const C *tw, cudaStream_t st, bool field, double *partials, int *nparts)
+{
+    if constexpr (sizeof(T) != 4) {
+        return cudaErrorNotSupported;
+    } else {
+        if ((L != 32 && L != 64 && L != 128) || !ntile || ((uintptr_t)ntile & 15) || nrows < 1 || 2 * nrows > L)
+            return cudaErrorNotSupported;
+        const int tc = zt_cols(L, Py, Kx), ntx = (Kx + tc - 1) / tc, grid = ntx * Py;
+        const int mode = !field ? ZT_ENERGY : (partials ? ZT_BOTH : ZT_FIELD);
+        if (nparts) {
+            if (partials && grid > *nparts) return cudaErrorNotSupported;
+            *nparts = partials ? grid : 0;
+        }
+#define DEMAG_ZT(LL, TC)                                                                                       \
+    if (L == LL && tc == TC) {                                                                                 \
+        using Sh = ZtShape<LL, TC>;                                                                            \
+        cudaError_t e;                                                                                         \
+        if (mode == ZT_FIELD) {                                                                                \
+            if ((e = allow_smem<k_z_t<LL, TC, ZT_FIELD>>(Sh::SMEM)) != cudaSuccess) return e;                  \
+            k_z_t<LL, TC, ZT_FIELD><<<grid, Sh::NT, Sh::SMEM, st>>>(S, Kx, Py, ss, rs, cs, nrows, ntile, tw, ntx, nullptr);   \
+        } else if (mode == ZT_ENERGY) {                                                                        \
+            if ((e = allow_smem<k_z_t<LL, TC, ZT_ENERGY>>(Sh::SMEM)) != cudaSuccess) return e;                 \
+            k_z_t<LL, TC, ZT_ENERGY><<<grid, Sh::NT, Sh::SMEM, st>>>(S, Kx, Py, ss, rs, cs, nrows, ntile, tw, ntx, partials); \
+        } else {                                                                                               \
+            if ((e = allow_smem<k_z_t<LL, TC, ZT_BOTH>>(Sh::SMEM)) != cudaSuccess) return e;                   \
+            k_z_t<LL, TC, ZT_BOTH><<<grid, Sh::NT, Sh::SMEM, st>>>(S, Kx, Py, ss, rs, cs, nrows, ntile, tw, ntx, partials);   \
+        }                                                                                                      \
+        return cudaGetLastError();                                                                             \
+    }
+        DEMAG_ZT(32, 16) DEMAG_ZT(32, 8) DEMAG_ZT(64, 8) DEMAG_ZT(128, 16) DEMAG_ZT(128, 8)
+#undef DEMAG_ZT
+        return cudaErrorNotSupported;
+    }
+}
+
+// Spectral-energy z pass of the two-stage kernel: FP64 plans take the 8-point second
+// stage (variant 8) for lengths 32..128, as in the field pipeline's fastest
+// form there; FP32 plans run k_z_t at these lengths.
 template <int L> constexpr int kZEnergyV = (L >= 32 && L <= 128) ? 8 : 0;
 
 template <typename T>
@@ -426,6 +492,7 @@ int Passes<T>::zenergy_blocks(int L, int Py, int Kx)
         }
         n = (ncols + tc - 1) / tc;
     }
+    if (sizeof(T) == 4 && L >= 32 && L <= 128) n = std::max(n, (Kx + 7) / 8 * Py);  // k_z_t at its narrowest tiles
     const int ws = 2 * sm_count();  // the persistent form: at most two CTAs per SM
     return n > ws ? n : ws;
 }
@@ -449,7 +516,7 @@ cudaError_t Passes<T>::zconv_energy(int L, C *S, int ncols, int width, int64_t s
     }
 #define DEMAG_CASE(LL)                                                                                     \
     case LL: {                                                                                             \
-        constexpr int V = kZEnergyV<LL>;                                                                   \
+        constexpr int V = sizeof(T) == 8 ? kZEnergyV<LL> : 0;                                              \
         using Sh = ZShape<T, LL, V>;                                                                       \
         const size_t sm = 3 * swsize(LL * Sh::TC) * sizeof(C) + (LL / 2 + 1) * 6 * Sh::TC * sizeof(T);     \
         cudaError_t e = allow_smem<k_z_energy2<T, LL, V>>(sm);                                             \
@@ -460,7 +527,9 @@ cudaError_t Passes<T>::zconv_energy(int L, C *S, int ncols, int width, int64_t s
                                                         twstride, partials);                              \
         return cudaGetLastError();                                                                         \
     }
-    switch (L) { DEMAG_CASE(32) DEMAG_CASE(64) DEMAG_CASE(128) DEMAG_CASE(256) DEMAG_CASE(512) default: return cudaErrorNotSupported; }
+    if constexpr (sizeof(T) == 8)
+        switch (L) { DEMAG_CASE(32) DEMAG_CASE(64) DEMAG_CASE(128) default: break; }
+    switch (L) { DEMAG_CASE(256) DEMAG_CASE(512) default: return cudaErrorNotSupported; }
 #undef DEMAG_CASE
 }
 
@@ -491,7 +560,17 @@ cudaError_t Passes<T>::x_fwd(int L, const XIn<T> &a, int nrows, int nvalid, C *o
         default: break;
         }
     }
-    if (L >= 64) {
+    if (L >= 16) {
+        // short rows: one-warp CTAs while the wide ones would leave SMs without work
+#define DEMAG_CASEN(LL)                                                                        \
+    if (L == LL && nvalid <= LL && (nrows + XShape<T, LL>::TR - 1) / XShape<T, LL>::TR < 2 * sm_count()) {     \
+        using S = XShape<T, LL, 32>;                                                           \
+        k_x_fwd2<T, LL, true, 32><<<(nrows + S::TR - 1) / S::TR, 32, (size_t)S::TR * S::RS * sizeof(C), st>>>( \
+            a, nrows, nvalid, out, out_rs, twx);                                               \
+        return cudaGetLastError();                                                             \
+    }
+        DEMAG_CASEN(16) DEMAG_CASEN(32) DEMAG_CASEN(64)
+#undef DEMAG_CASEN
 #define DEMAG_CASE2(LL)                                                                        \
     case LL: {                                                                                 \
         using S = XShape<T, LL>;                                                               \
@@ -503,34 +582,42 @@ cudaError_t Passes<T>::x_fwd(int L, const XIn<T> &a, int nrows, int nvalid, C *o
             k_x_fwd2<T, LL, false><<<grid, S::NT, sm, st>>>(a, nrows, nvalid, out, out_rs, twx); \
         return cudaGetLastError();                                                             \
     }
-        switch (L) { DEMAG_CASE2(64) DEMAG_CASE2(128) DEMAG_CASE2(256) DEMAG_CASE2(512) default: return cudaErrorInvalidValue; }
+        switch (L) { DEMAG_CASE2(16) DEMAG_CASE2(32) DEMAG_CASE2(64) DEMAG_CASE2(128) DEMAG_CASE2(256) DEMAG_CASE2(512) default: return cudaErrorInvalidValue; }
 #undef DEMAG_CASE2
     }
 #define DEMAG_CASE(LL)                                                                        \
     case LL: {                                                                                \
-        if constexpr (LL <= 512) {                                                            \
-            using S = TileShape<T, LL>;                                                       \
-            const size_t sm = swsize(LL * S::TC) * sizeof(C);                                 \
-            cudaError_t e = allow_smem<k_x_fwd<T, LL>>(sm);                                   \
-            if (e != cudaSuccess) return e;                                                   \
-            const int grid = (nrows + S::TC - 1) / S::TC;                                     \
-            k_x_fwd<T, LL><<<grid, S::NT, sm, st>>>(a, nrows, nvalid, out, out_rs, twx); \
-            return cudaGetLastError();                                                        \
-        } else {                                                                              \
-            return cudaErrorInvalidValue;                                                     \
-        }                                                                                     \
+        using S = TileShape<T, LL>;                                                           \
+        const size_t sm = swsize(LL * S::TC) * sizeof(C);                                     \
+        cudaError_t e = allow_smem<k_x_fwd<T, LL>>(sm);                                       \
+        if (e != cudaSuccess) return e;                                                       \
+        const int grid = (nrows + S::TC - 1) / S::TC;                                         \
+        k_x_fwd<T, LL><<<grid, S::NT, sm, st>>>(a, nrows, nvalid, out, out_rs, twx);          \
+        return cudaGetLastError();                                                            \
     }
-    switch (L) { DEMAG_FOR_EACH_L(DEMAG_CASE) default: return cudaErrorInvalidValue; }
+    switch (L) { DEMAG_CASE(1) DEMAG_CASE(2) DEMAG_CASE(4) DEMAG_CASE(8) default: return cudaErrorInvalidValue; }
 #undef DEMAG_CASE
 }
 
+// Whether the one-tile inverse x pass (not the pipelined form of variant 2, L >= 64)
+// runs its one-warp CTAs (see x_inv).
 template <typename T>
-int Passes<T>::x_blocks(int L, int nrows)
+static bool x_inv_narrow(int L, int nrows)
+{
+    const int tr = L == 16 ? XShape<T, 16>::TR : L == 32 ? XShape<T, 32>::TR : L == 64 ? XShape<T, 64>::TR : 0;
+    return tr && (nrows + tr - 1) / tr < 2 * sm_count();
+}
+
+template <typename T>
+int Passes<T>::x_blocks(int L, int nrows, int variant)
 {
     if (!pow2_len(L)) return MixedPasses<T>::x_blocks(L, nrows);
     int rows_per_cta;
+    const bool nw = x_inv_narrow<T>(L, nrows) && !(variant == 2 && L >= 64);
     switch (L) {
-    case 64: rows_per_cta = XShape<T, 64>::TR; break;
+    case 16: rows_per_cta = nw ? XShape<T, 16, 32>::TR : XShape<T, 16>::TR; break;
+    case 32: rows_per_cta = nw ? XShape<T, 32, 32>::TR : XShape<T, 32>::TR; break;
+    case 64: rows_per_cta = nw ? XShape<T, 64, 32>::TR : XShape<T, 64>::TR; break;
     case 128: rows_per_cta = XShape<T, 128>::TR; break;
     case 256: rows_per_cta = XShape<T, 256>::TR; break;
     case 512: rows_per_cta = XShape<T, 512>::TR; break;
@@ -556,7 +643,21 @@ cudaError_t Passes<T>::x_inv(int L, const C *in, int64_t in_rs, int nrows, int n
         switch (L) { DEMAG_PIPE(64) DEMAG_PIPE(128) DEMAG_PIPE(256) default: break; }
 #undef DEMAG_PIPE
     }
-    if (L >= 64) {
+    if (L >= 16) {
+        if (x_inv_narrow<T>(L, nrows)) {
+#define DEMAG_CASEN(LL)                                                                        \
+    if (L == LL) {                                                                             \
+        using S = XShape<T, LL, 32>;                                                           \
+        const size_t sm = (size_t)S::TR * S::RS * sizeof(C);                                   \
+        const int grid = (nrows + S::TR - 1) / S::TR;                                          \
+        if (nvalid <= LL) k_x_inv2<T, LL, false, false, 32><<<grid, 32, sm, st>>>(in, in_rs, nrows, nvalid, o, twx); \
+        else if (nvalid == LL + 1) k_x_inv2<T, LL, true, false, 32><<<grid, 32, sm, st>>>(in, in_rs, nrows, nvalid, o, twx); \
+        else return cudaErrorInvalidValue;                                                     \
+        return cudaGetLastError();                                                             \
+    }
+            DEMAG_CASEN(16) DEMAG_CASEN(32) DEMAG_CASEN(64)
+#undef DEMAG_CASEN
+        }
 #define DEMAG_CASE2(LL)                                                                        \
     case LL: {                                                                                 \
         using S = XShape<T, LL>;                                                               \
@@ -573,24 +674,20 @@ cudaError_t Passes<T>::x_inv(int L, const C *in, int64_t in_rs, int nrows, int n
         else return cudaErrorInvalidValue;                                                     \
         return cudaGetLastError();                                                             \
     }
-        switch (L) { DEMAG_CASE2(64) DEMAG_CASE2(128) DEMAG_CASE2(256) DEMAG_CASE2(512) default: return cudaErrorInvalidValue; }
+        switch (L) { DEMAG_CASE2(16) DEMAG_CASE2(32) DEMAG_CASE2(64) DEMAG_CASE2(128) DEMAG_CASE2(256) DEMAG_CASE2(512) default: return cudaErrorInvalidValue; }
 #undef DEMAG_CASE2
     }
 #define DEMAG_CASE(LL)                                                                        \
     case LL: {                                                                                \
-        if constexpr (LL <= 512) {                                                            \
-            using S = TileShape<T, LL>;                                                       \
-            const size_t sm = swsize(LL * S::TC) * sizeof(C);                                 \
-            cudaError_t e = allow_smem<k_x_inv<T, LL>>(sm);                                   \
-            if (e != cudaSuccess) return e;                                                   \
-            const int grid = (nrows + S::TC - 1) / S::TC;                                     \
-            k_x_inv<T, LL><<<grid, S::NT, sm, st>>>(in, in_rs, nrows, nvalid, o, twx);           \
-            return cudaGetLastError();                                                        \
-        } else {                                                                              \
-            return cudaErrorInvalidValue;                                                     \
-        }                                                                                     \
+        using S = TileShape<T, LL>;                                                           \
+        const size_t sm = swsize(LL * S::TC) * sizeof(C);                                     \
+        cudaError_t e = allow_smem<k_x_inv<T, LL>>(sm);                                       \
+        if (e != cudaSuccess) return e;                                                       \
+        const int grid = (nrows + S::TC - 1) / S::TC;                                         \
+        k_x_inv<T, LL><<<grid, S::NT, sm, st>>>(in, in_rs, nrows, nvalid, o, twx);            \
+        return cudaGetLastError();                                                            \
     }
-    switch (L) { DEMAG_FOR_EACH_L(DEMAG_CASE) default: return cudaErrorInvalidValue; }
+    switch (L) { DEMAG_CASE(1) DEMAG_CASE(2) DEMAG_CASE(4) DEMAG_CASE(8) default: return cudaErrorInvalidValue; }
 #undef DEMAG_CASE
 }
 
@@ -763,14 +860,14 @@ cudaError_t Passes<T>::zconv(int L, C *S, int ncols, int width, int64_t ss, int6
              : variant == 2 ? zconv_launch<LL, 2>(S, ncols, width, ss, rs, cs, nrows, nhat, Py, Kx, tw, twstride, st) \
              : variant == 4 ? zconv_launch<LL, 4>(S, ncols, width, ss, rs, cs, nrows, nhat, Py, Kx, tw, twstride, st) \
                             : zconv_launch<LL, 0>(S, ncols, width, ss, rs, cs, nrows, nhat, Py, Kx, tw, twstride, st);
-    if (variant == 8) {  // 8-point second stage, two CTAs per SM (lengths 32..128)
-        switch (L) {
+    // 8-point second stage, two CTAs per SM (lengths 32..128; FP32 plans run k_z_t for it)
+    if constexpr (sizeof(T) == 8)
+        if (variant == 8) switch (L) {
         case 32: return zconv_launch<32, 8>(S, ncols, width, ss, rs, cs, nrows, nhat, Py, Kx, tw, twstride, st);
         case 64: return zconv_launch<64, 8>(S, ncols, width, ss, rs, cs, nrows, nhat, Py, Kx, tw, twstride, st);
         case 128: return zconv_launch<128, 8>(S, ncols, width, ss, rs, cs, nrows, nhat, Py, Kx, tw, twstride, st);
-        default: variant = 0;
+        default: break;
         }
-    }
     switch (L) { DEMAG_CASE(32) DEMAG_CASE(64) DEMAG_CASE(128) DEMAG_CASE(256) DEMAG_CASE(512) default: return cudaErrorInvalidValue; }
 #undef DEMAG_CASE
 }
@@ -778,11 +875,19 @@ cudaError_t Passes<T>::zconv(int L, C *S, int ncols, int width, int64_t ss, int6
 template <typename T>
 cudaError_t Passes<T>::sp_zconv(int L, C *S, int ncols, int width, int64_t ss, int64_t rs, int64_t cs, int nrows,
                                 int nout, const T *that, int Py, int Kx, const C *tw, const C *phx, const C *phy,
-                                const C *phz, cudaStream_t st, int variant)
+                                const C *phz, cudaStream_t st, int variant, const T *ttile)
 {
     if (ncols <= 0) return cudaSuccess;
     // zero padding: nz + 1 node rows out of L >= 2 nz
     if (L < 2 || 2 * nrows > L || nout != nrows + 1 || cs != (int64_t)nrows * rs) return cudaErrorInvalidValue;
+    if constexpr (sizeof(T) == 4) {
+        // the persistent form, where the plan has its tables
+        if (width == Kx && ncols == Py * Kx && zws_ok(L, S, ttile, nrows, ss, rs, cs, sizeof(C))) {
+            const cudaError_t e = L == 256 ? spws_launch<256>(S, Kx, Py, ss, rs, cs, nrows, nout, ttile, tw, phx, phy, phz, st)
+                                           : spws_launch<512>(S, Kx, Py, ss, rs, cs, nrows, nout, ttile, tw, phx, phy, phz, st);
+            if (e != cudaErrorNotSupported) return e;
+        }
+    }
     if (!pow2_len(L))
         return MixedPasses<T>::sp_zconv(L, S, ncols, width, ss, rs, cs, nrows, nout, that, Py, Kx, tw, phx, phy, phz, st);
     if (variant == 5) {
@@ -791,7 +896,10 @@ cudaError_t Passes<T>::sp_zconv(int L, C *S, int ncols, int width, int64_t ss, i
         case 32: e = sp_zconv_tma<T, 32>(S, ncols, width, ss, rs, cs, nrows, nout, that, Py, Kx, tw, phx, phy, phz, st); break;
         case 64: e = sp_zconv_tma<T, 64>(S, ncols, width, ss, rs, cs, nrows, nout, that, Py, Kx, tw, phx, phy, phz, st); break;
         case 128: e = sp_zconv_tma<T, 128>(S, ncols, width, ss, rs, cs, nrows, nout, that, Py, Kx, tw, phx, phy, phz, st); break;
-        case 256: e = sp_zconv_tma<T, 256>(S, ncols, width, ss, rs, cs, nrows, nout, that, Py, Kx, tw, phx, phy, phz, st); break;
+        case 256:
+            if constexpr (sizeof(T) == 8)
+                e = sp_zconv_tma<T, 256>(S, ncols, width, ss, rs, cs, nrows, nout, that, Py, Kx, tw, phx, phy, phz, st);
+            break;
         default: break;
         }
         if (e != cudaErrorNotSupported) return e;

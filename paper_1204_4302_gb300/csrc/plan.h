@@ -78,7 +78,8 @@ template <typename T> struct Passes {
                              const C *twx, cudaStream_t st, int variant = 0);
     // 1 if a bounded wait of a pipelined pass gave up since the last call (clears it)
     static int pipe_error_take();
-    static int x_blocks(int L, int nrows);
+    // CTAs (energy partials) of the inverse x pass; the largest is variant 0's
+    static int x_blocks(int L, int nrows, int variant = 0);
     // strided column transforms (y passes, z forward of the setup)
     static cudaError_t col(int L, bool inv, const C *in, C *out, int ncols, int width, int64_t iss,
                            int64_t irs, int nin, int64_t oss, int64_t ors, int nout, const C *tw,
@@ -101,6 +102,12 @@ template <typename T> struct Passes {
     static cudaError_t zconv_ws(int L, C *S, int Kx, int Py, int64_t ss, int64_t rs, int64_t cs, int nrows,
                                 const T *ntile, const C *tw, cudaStream_t st, int tc = 8,
                                 double *partials = nullptr, int *nparts = nullptr);
+    // z pass of small tiles (FP32, L = 32, 64 or 128) from the tile-ordered tensor
+    // copy: the field, with partials the spectral energy's sums too (as zconv_ws), or
+    // (field false) only these. cudaErrorNotSupported as for zconv_ws.
+    static cudaError_t zconv_t(int L, C *S, int Kx, int Py, int64_t ss, int64_t rs, int64_t cs, int nrows, const T *ntile,
+                               const C *tw, cudaStream_t st, bool field, double *partials = nullptr,
+                               int *nparts = nullptr);
     // spectral energy (the Parseval form of E, no inverse passes): forward z
     // transforms and the per-CTA sums of w(kx) m^H N^ m into partials
     // (*nparts of them; for zconv_ws_energy *nparts also holds the room in
@@ -115,9 +122,10 @@ template <typename T> struct Passes {
                                     double *partials, int *nparts, cudaStream_t st);
     // partial sums the spectral energy may write (0: no spectral form for L)
     static int zenergy_blocks(int L, int Py, int Kx);
-    // elements of the tile-ordered tensor copy for zconv_ws (0: not used for this L)
-    static size_t tile_tensor_elems(int L, int Py, int Kx);
-    static cudaError_t tile_tensor(int L, const T *nhat, T *ntile, int Py, int Kx, cudaStream_t st);
+    // elements of the tile-ordered copy of the tensor (zconv_ws, zconv_t, the
+    // mixed-radix z pass) or of the SP kernel tables (sp); 0: not used for this L
+    static size_t tile_tensor_elems(int L, int Py, int Kx, bool sp);
+    static cudaError_t tile_tensor(int L, const T *nhat, T *ntile, int Py, int Kx, cudaStream_t st, bool sp);
     template <int L>
     static cudaError_t zconv_pipe(C *S, int ncols, int width, int64_t ss, int64_t rs, int64_t cs, int nrows,
                                   const T *nhat, int Py, int Kx, const C *tw, int twstride, cudaStream_t st);
@@ -131,7 +139,8 @@ template <typename T> struct Passes {
     // spectrum out, nout = nz + 1 node rows) and the finite-difference field
     static cudaError_t sp_zconv(int L, C *S, int ncols, int width, int64_t ss, int64_t rs, int64_t cs,
                                 int nrows, int nout, const T *that, int Py, int Kx, const C *tw,
-                                const C *phx, const C *phy, const C *phz, cudaStream_t st, int variant = 0);
+                                const C *phx, const C *phy, const C *phz, cudaStream_t st, int variant = 0,
+                                const T *ttile = nullptr);
     static cudaError_t sp_grad(const T *phi, int nx, int ny, int nz, double dx, double dy, double dz, T *H,
                                const T *Mref, double *partials, cudaStream_t st);
     static int sp_grad_blocks(int nx, int ny, int nz);
@@ -144,12 +153,17 @@ struct BatchState {
     float *H;
     float2 *S1, *S2;
     const float *nhat;
+    const float *ntile;  // tile-ordered tensor copy (z lengths 32..128: k_z_t)
     const float2 *tw[3];
     double *partials;
     double *E;
     int nx, ny, nz, Px, Py, Pz, Kx, Kxp;
     int ntiles[6];  // tiles of each pass (x fwd, y fwd, z, y inv, x inv, energy)
     double efactor; // -(mu0/2) V
+    // the energy's spectral sum taken in the z tiles (z lengths 32..128): their
+    // number (0: taken in the x inverse pass) and (mu0/2) V / (Px Py Pz)
+    int nez;
+    double ezfactor;
 };
 
 // Shared description of one batch launch (kernel argument).

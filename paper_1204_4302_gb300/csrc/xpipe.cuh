@@ -9,6 +9,7 @@
 #include <cuda.h>  // CUtensorMap (the map is built on the host, see passes_impl.cuh)
 
 #include "fft2.cuh"
+#include "sp.cuh"
 
 namespace demag {
 
@@ -181,8 +182,7 @@ k_x_fwd_tma(const T *__restrict__ in, T wscalar, int nrows, int nvalid, typename
                 for (int r = 0; r < R1 / 2; ++r) {
                     const int x0 = 2 * (j1 + r * R2);
                     if (x0 < nvalid) {  // nvalid is even
-                        const C q = *reinterpret_cast<const C *>(p + x0);
-                        u[r] = cmk<C>(q.x * wscalar, q.y * wscalar);
+                        u[r] = cscale_rn(*reinterpret_cast<const C *>(p + x0), wscalar);
                     }
                 }
             }

@@ -296,18 +296,18 @@ template <int L, int TC> struct ZwsShape {
 };
 
 // Tile-ordered copy of the FP32 octant tensor spectrum for the persistent z
-// pass: [Py/2+1][ntx4][6][Pz/2+1][4] (4-column sub-blocks, ntx4 = ceil(Kx/4)
+// pass: [Py/2+1][ntx4][NC][Pz/2+1][4] (4-column sub-blocks, ntx4 = ceil(Kx/4)
 // rounded up to even), zero for kx >= Kx; each sub-block is contiguous and
-// fetched with one bulk copy.
-template <typename T>
+// fetched with one bulk copy. NC: 6 tensor components, or the 3 kernel tables of SP.
+template <typename T, int NC>
 __global__ void k_tile_tensor(const T *__restrict__ nhat, T *__restrict__ out, int Kx, int hy, int HZ, int ntx4)
 {
-    const int64_t total = (int64_t)hy * ntx4 * 6 * HZ * 4;
+    const int64_t total = (int64_t)hy * ntx4 * NC * HZ * 4;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         int64_t r = i;
         const int c = (int)(r & 3); r >>= 2;
         const int kzf = (int)(r % HZ); r /= HZ;
-        const int comp = (int)(r % 6); r /= 6;
+        const int comp = (int)(r % NC); r /= NC;
         const int kxt = (int)(r % ntx4);
         const int kyf = (int)(r / ntx4);
         const int kx = kxt * 4 + c;
