@@ -80,20 +80,34 @@ __global__ void k_tg_tables(const double *__restrict__ snode, int R, int nx, int
     }
 }
 
-// Factor transform on axis q: out[v][i] = sum_j D[i - j] u[v][j] for the
-// vectors v = (l, p, m) (K = 3 R r of them), D the plain table (p != q) or
-// the odd one (p = q) of node l. On axis x the weight W_l lam_m^(p) / (4 pi)
-// is folded in. One block per (l, p): its r vectors share the table, so a
-// thread (output i) takes each table entry once for VC vectors at a time
-// (VC = 8, 4, 2 or 1 by the rank), whose factors sit in shared memory as
-// [j][VC] (read two at a time).
+// Factor transforms: on axis q, out[v][i] = sum_j D[i - j] u[v][j] for the
+// vectors v = (l, p, m) (3 R r_q of them), D the plain table (p != q) or the odd one
+// (p = q) of node l. On axis x the weight W_l lam_m^(p) / (4 pi) is folded in.
+// One launch for the three axes, a block per (l, p) and axis: its r vectors share
+// the table in shared memory, VC of them at a time with their factors as [j][VC].
+// What bounds it is shared-memory reads per multiply-add, so a thread forms
+// kTgNO outputs (a block's width apart: consecutive lanes read consecutive table
+// entries) of the VC vectors: kTgNO table reads and VC / 4 vector reads for
+// kTgNO VC multiply-adds. Rank 8 at 256^3: 52 us for three launches of one output per
+// thread (9 reads for 8 multiply-adds).
+constexpr int kTgNO = 4;
+template <typename T> struct TgAxes {
+    const T *U[3];
+    T *out[3];
+    int n[3], r[3];
+};
+
 template <typename T, int VC>
-__global__ void __launch_bounds__(512)
-k_tg_apply(const T *__restrict__ tab, int tstride, const T *__restrict__ U, const T *__restrict__ lam,
-           const double *__restrict__ wnode, int R, int r, int q, int n, T *__restrict__ out)
+__global__ void __launch_bounds__(128)
+k_tg_apply(const T *__restrict__ tab, int tstride, const T *__restrict__ lam, const double *__restrict__ wnode, int R,
+           const TgAxes<T> ax)
 {
-    using V2 = typename CplxOf<T>::type;  // two values (float2 / double2)
+    constexpr int W = VC < 4 ? VC : 4;  // values per vector read
+    struct alignas(W * sizeof(T) < 16 ? W * sizeof(T) : 16) Vec { T v[W]; };
     extern __shared__ __align__(16) unsigned char smraw[];
+    const int q = blockIdx.y, n = ax.n[q], r = ax.r[q];
+    const T *__restrict__ U = ax.U[q];
+    T *__restrict__ out = ax.out[q];
     T *su = reinterpret_cast<T *>(smraw);   // [n][VC]
     T *st = su + (size_t)n * VC;             // [2n - 1]
     const int lp = blockIdx.x;               // l * 3 + p
@@ -104,51 +118,65 @@ k_tg_apply(const T *__restrict__ tab, int tstride, const T *__restrict__ U, cons
         const int mc = min(VC, r - m0);
         __syncthreads();  // the previous chunk's factors are read
         for (int e = threadIdx.x; e < n * VC; e += blockDim.x) {
-            const int j = e / VC, mm = e % VC;
-            su[e] = mm < mc ? U[((int64_t)p * r + m0 + mm) * n + j] : (T)0;
+            const int mm = e / n, j = e - mm * n;
+            su[j * VC + mm] = mm < mc ? U[((int64_t)p * r + m0 + mm) * n + j] : (T)0;
         }
         __syncthreads();
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            T acc[VC];
+        for (int i0 = threadIdx.x; i0 < n; i0 += kTgNO * blockDim.x) {
+            T acc[kTgNO][VC];
+            const T *d[kTgNO];
 #pragma unroll
-            for (int mm = 0; mm < VC; ++mm) acc[mm] = 0;
+            for (int o = 0; o < kTgNO; ++o) {
+                // an output past the row reads the last one's table entries and is dropped
+                d[o] = st + min(i0 + o * (int)blockDim.x, n - 1) + n - 1;
+#pragma unroll
+                for (int mm = 0; mm < VC; ++mm) acc[o][mm] = 0;
+            }
             for (int j = 0; j < n; ++j) {
-                const T d = st[i - j + n - 1];
-                if constexpr (VC == 1) {
-                    acc[0] += d * su[j];
-                } else {
-                    const V2 *f = reinterpret_cast<const V2 *>(su + (size_t)j * VC);
+                T f[VC];
 #pragma unroll
-                    for (int h = 0; h < VC / 2; ++h) {
-                        const V2 w = f[h];
-                        acc[2 * h] += d * w.x;
-                        acc[2 * h + 1] += d * w.y;
-                    }
+                for (int h = 0; h < VC / W; ++h) {
+                    const Vec w = reinterpret_cast<const Vec *>(su + (size_t)j * VC)[h];
+#pragma unroll
+                    for (int e = 0; e < W; ++e) f[h * W + e] = w.v[e];
+                }
+#pragma unroll
+                for (int o = 0; o < kTgNO; ++o) {
+                    const T dv = d[o][-j];
+#pragma unroll
+                    for (int mm = 0; mm < VC; ++mm) acc[o][mm] += dv * f[mm];
                 }
             }
-            for (int mm = 0; mm < mc; ++mm) {
-                const int m = m0 + mm, v = lp * r + m;
-                T scale = (T)1;
-                if (q == 0) scale = (T)(wnode[l] * (double)lam[p * r + m] * (1.0 / (4.0 * 3.14159265358979323846)));
-                out[(int64_t)v * n + i] = acc[mm] * scale;
+#pragma unroll
+            for (int o = 0; o < kTgNO; ++o) {
+                const int i = i0 + o * (int)blockDim.x;
+                if (i >= n) continue;
+                for (int mm = 0; mm < mc; ++mm) {
+                    const int m = m0 + mm, v = lp * r + m;
+                    T scale = (T)1;
+                    if (q == 0) scale = (T)(wnode[l] * (double)lam[p * r + m] * (1.0 / (4.0 * 3.14159265358979323846)));
+                    out[(int64_t)v * n + i] = acc[o][mm] * scale;
+                }
             }
         }
     }
 }
 
 template <typename T>
-void tg_apply(const T *tab, int tstride, const T *U, const T *lam, const double *wnode, int R, int r, int q, int n,
-              T *out, cudaStream_t st)
+cudaError_t tg_apply(const T *tab, int tstride, const TgAxes<T> &ax, const T *lam, const double *wnode, int R, cudaStream_t st)
 {
-    const int threads = n >= 512 ? 512 : ((n + 31) / 32) * 32;
+    const int n = std::max(ax.n[0], std::max(ax.n[1], ax.n[2])), r = std::max(ax.r[0], std::max(ax.r[1], ax.r[2]));
+    const int threads = std::min(128, (n + 32 * kTgNO - 1) / (32 * kTgNO) * 32);
     const int vc = r >= 8 ? 8 : (r >= 4 ? 4 : (r >= 2 ? 2 : 1));
     const size_t sm = (size_t)(vc * n + 2 * n) * sizeof(T);
+    const dim3 grid(3 * R, 3);
     switch (vc) {
-    case 8: k_tg_apply<T, 8><<<3 * R, threads, sm, st>>>(tab, tstride, U, lam, wnode, R, r, q, n, out); break;
-    case 4: k_tg_apply<T, 4><<<3 * R, threads, sm, st>>>(tab, tstride, U, lam, wnode, R, r, q, n, out); break;
-    case 2: k_tg_apply<T, 2><<<3 * R, threads, sm, st>>>(tab, tstride, U, lam, wnode, R, r, q, n, out); break;
-    default: k_tg_apply<T, 1><<<3 * R, threads, sm, st>>>(tab, tstride, U, lam, wnode, R, r, q, n, out); break;
+    case 8: k_tg_apply<T, 8><<<grid, threads, sm, st>>>(tab, tstride, lam, wnode, R, ax); break;
+    case 4: k_tg_apply<T, 4><<<grid, threads, sm, st>>>(tab, tstride, lam, wnode, R, ax); break;
+    case 2: k_tg_apply<T, 2><<<grid, threads, sm, st>>>(tab, tstride, lam, wnode, R, ax); break;
+    default: k_tg_apply<T, 1><<<grid, threads, sm, st>>>(tab, tstride, lam, wnode, R, ax); break;
     }
+    return cudaGetLastError();
 }
 
 // Dense block-CP contraction Phi[k][j][i] = sum_K Z[K][k] Y[K][j] X[K][i].
@@ -215,8 +243,15 @@ k_tg_dense(const T *__restrict__ X, const T *__restrict__ Y, const T *__restrict
 
 // Second-order differences of the cell-centre potential (central inside,
 // one-sided at the ends; n >= 3 per axis), H = -grad Phi, and optionally the
-// energy partials sum over the block of M . H with M rebuilt from its factors.
-constexpr int kTgFieldThreads = 128;
+// energy partials sum over the block of M . H with M rebuilt from its factors,
+// M^(p)[k][j][i] = sum_m w[p r + m] Ux[p r + m][i], the row-constant part w in shared
+// memory (CP: w = lam Uy[j] Uz[k]; Tucker, G given: w[p r + a] = sum_{b,c} G B[b][j]
+// C[c][k] with r = r1).
+// The energy's 3 r loads and multiply-adds per cell bound it, so a block takes
+// kTgFieldRows rows j at once and a thread one i of all of them: a factor is loaded
+// once for four cells, their w arrive in one vector read, and the rows share their y
+// neighbours. Rank 8 at 256^3: 202 us with one row at a time.
+constexpr int kTgFieldThreads = 128, kTgFieldRows = 4;
 
 template <typename T>
 __global__ void __launch_bounds__(kTgFieldThreads)
@@ -224,73 +259,101 @@ k_tg_field(const T *__restrict__ phi, int nx, int ny, int nz, T hx, T hy, T hz, 
            const T *__restrict__ lam, const T *__restrict__ Ux, const T *__restrict__ Uy, const T *__restrict__ Uz, int r,
            double *__restrict__ partials, const T *__restrict__ G = nullptr, int r2 = 0, int r3 = 0)
 {
-    // One block per x row (j, k) at a time (grid-stride over rows), threads
-    // over i. The energy's M^(p)[k][j][i] = sum_m w[p r + m] Ux[p r + m][i]
-    // takes the row-constant part from shared memory (CP: w = lam Uy[j]
-    // Uz[k]; Tucker, G given: w[p r + a] = sum_{b,c} G B[b][j] C[c][k] with
-    // r = r1), so a cell costs 3 r coalesced factor loads and no index
-    // divisions; the energy leaves one FP64 partial per block.
-    __shared__ T w[3 * 64];
-    __shared__ double ws[kTgFieldThreads / 32];
+    constexpr int JR = kTgFieldRows;
+    struct alignas(16) Row4 { T v[JR]; };
+    __shared__ Row4 w[3 * 64];
     const int64_t sy = nx, sz = (int64_t)nx * ny, ncell = sz * nz;
     const T ix = (T)0.5 / hx, iy = (T)0.5 / hy, iz = (T)0.5 / hz;
-    const int nrows = ny * nz;
+    const int jg = (ny + JR - 1) / JR, ngroups = jg * nz;
     T acc = 0;
-    for (int row = blockIdx.x; row < nrows; row += gridDim.x) {
-        const int j = row % ny, k = row / ny;
+    for (int grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
+        const int k = grp / jg, j0 = (grp - k * jg) * JR, rows = min(JR, ny - j0);
         if (partials) {
-            __syncthreads();  // the previous row's w is read
-            if (G) {
-                // Tucker: w[p r + a] = sum_{b,c} G^(p)[c][b][a] B^(p)[b][j] C^(p)[c][k]
-                for (int v = threadIdx.x; v < 3 * r; v += blockDim.x) {
-                    const int p = v / r, a = v % r;
-                    const T *Gp = G + (int64_t)p * r3 * r2 * r;
-                    T acc = 0;
-                    for (int c = 0; c < r3; ++c) {
-                        T t = 0;
-                        for (int b = 0; b < r2; ++b) t += Gp[(c * r2 + b) * r + a] * Uy[(p * r2 + b) * ny + j];
-                        acc += t * Uz[(p * r3 + c) * nz + k];
+            __syncthreads();  // the previous group's w is read
+            for (int e = threadIdx.x; e < 3 * r * JR; e += blockDim.x) {
+                const int v = e / JR, q = e % JR, j = j0 + q;
+                T x = 0;
+                if (q < rows) {
+                    if (G) {
+                        const int p = v / r, a = v % r;
+                        const T *Gp = G + (int64_t)p * r3 * r2 * r;
+                        for (int c = 0; c < r3; ++c) {
+                            T t = 0;
+                            for (int b = 0; b < r2; ++b) t += Gp[(c * r2 + b) * r + a] * Uy[(p * r2 + b) * ny + j];
+                            x += t * Uz[(p * r3 + c) * nz + k];
+                        }
+                    } else {
+                        x = lam[v] * Uy[v * ny + j] * Uz[v * nz + k];
                     }
-                    w[v] = acc;
                 }
-            } else {
-                for (int v = threadIdx.x; v < 3 * r; v += blockDim.x) w[v] = lam[v] * Uy[v * ny + j] * Uz[v * nz + k];
+                w[v].v[q] = x;  // zero in rows past ny
             }
             __syncthreads();
         }
-        const T *prow = phi + (int64_t)row * nx;
-        // y and z differences: central inside, one-sided at the ends
-        const int64_t jm = j == 0 ? 0 : (j == ny - 1 ? -2 * sy : -sy), jp = j == 0 ? 2 * sy : (j == ny - 1 ? 0 : sy);
+        // z neighbours: central inside, one-sided at the ends
         const int64_t km = k == 0 ? 0 : (k == nz - 1 ? -2 * sz : -sz), kp = k == 0 ? 2 * sz : (k == nz - 1 ? 0 : sz);
+        const bool kend = k == 0 || k == nz - 1;
+        const int64_t kc = k == 0 ? sz : -sz;
+        const T ks = k == 0 ? (T)1 : (T)-1;  // one-sided: ks (4 f[kc] - 3 f[0] - f[far])
         for (int i = threadIdx.x; i < nx; i += blockDim.x) {
-            const T *f = prow + i;
-            T d0, d1, d2;
-            if (i == 0) d0 = ((T)-3 * f[0] + (T)4 * f[1] - f[2]) * ix;
-            else if (i == nx - 1) d0 = ((T)3 * f[0] - (T)4 * f[-1] + f[-2]) * ix;
-            else d0 = (f[1] - f[-1]) * ix;
-            if (j == 0) d1 = ((T)-3 * f[0] + (T)4 * f[sy] - f[jp]) * iy;
-            else if (j == ny - 1) d1 = ((T)3 * f[0] - (T)4 * f[-sy] + f[jm]) * iy;
-            else d1 = (f[jp] - f[jm]) * iy;
-            if (k == 0) d2 = ((T)-3 * f[0] + (T)4 * f[sz] - f[kp]) * iz;
-            else if (k == nz - 1) d2 = ((T)3 * f[0] - (T)4 * f[-sz] + f[km]) * iz;
-            else d2 = (f[kp] - f[km]) * iz;
-            const int64_t c = (int64_t)row * nx + i;
+            const T *f = phi + ((int64_t)k * ny + j0) * nx + i;
+            // rows j0 - 2 .. j0 + JR of this column (the outermost only where a one-sided difference needs it)
+            T c[JR + 3];
+#pragma unroll
+            for (int q = -2; q <= JR; ++q) {
+                const bool need = j0 + q >= 0 && j0 + q < ny && (q > -2 || rows == 1) && (q <= rows || (q == 2 && rows == 1));
+                c[q + 2] = need ? f[q * sy] : (T)0;
+            }
+            T d[JR][3];
+#pragma unroll
+            for (int q = 0; q < JR; ++q) {
+                d[q][0] = d[q][1] = d[q][2] = 0;
+                if (q >= rows) continue;
+                const T *g = f + q * sy;
+                const T f0 = c[q + 2];
+                if (i == 0) d[q][0] = ((T)-3 * f0 + (T)4 * g[1] - g[2]) * ix;
+                else if (i == nx - 1) d[q][0] = ((T)3 * f0 - (T)4 * g[-1] + g[-2]) * ix;
+                else d[q][0] = (g[1] - g[-1]) * ix;
+                const int j = j0 + q;
+                if (j == 0) d[q][1] = ((T)-3 * f0 + (T)4 * c[q + 3] - (q + 4 < JR + 3 ? c[q + 4] : (T)0)) * iy;
+                else if (j == ny - 1) d[q][1] = ((T)3 * f0 - (T)4 * c[q + 1] + c[q]) * iy;
+                else d[q][1] = (c[q + 3] - c[q + 1]) * iy;
+                const T zm = g[km], zp = g[kp];
+                if (kend) d[q][2] = ks * ((T)4 * g[kc] - (T)3 * f0 - (k == 0 ? zp : zm)) * iz;
+                else d[q][2] = (zp - zm) * iz;
+            }
             if (H) {
-                H[c] = -d0;
-                H[ncell + c] = -d1;
-                H[2 * ncell + c] = -d2;
+                T *h = H + ((int64_t)k * ny + j0) * nx + i;
+#pragma unroll
+                for (int q = 0; q < JR; ++q)
+                    if (q < rows) {
+                        h[q * sy] = -d[q][0];
+                        h[ncell + q * sy] = -d[q][1];
+                        h[2 * ncell + q * sy] = -d[q][2];
+                    }
             }
             if (partials) {
-                const T hv[3] = {-d0, -d1, -d2};
+#pragma unroll
                 for (int p = 0; p < 3; ++p) {
-                    T mp = 0;
-                    for (int m = 0; m < r; ++m) mp += w[p * r + m] * Ux[(p * r + m) * nx + i];
-                    acc += mp * hv[p];
+                    T m4[JR];
+#pragma unroll
+                    for (int q = 0; q < JR; ++q) m4[q] = 0;
+                    const T *u = Ux + (int64_t)p * r * nx + i;
+                    const Row4 *wp = w + p * r;
+                    for (int m = 0; m < r; ++m) {
+                        const T x = u[(int64_t)m * nx];
+                        const Row4 ww = wp[m];
+#pragma unroll
+                        for (int q = 0; q < JR; ++q) m4[q] += ww.v[q] * x;
+                    }
+#pragma unroll
+                    for (int q = 0; q < JR; ++q) acc -= m4[q] * d[q][p];
                 }
             }
         }
     }
     if (partials) {
+        __shared__ double ws[kTgFieldThreads / 32];
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = (double)acc;
         __syncthreads();
@@ -447,11 +510,16 @@ demag_status tg_run(demag_tg_plan *p, const void *lam, const void *Ux, const voi
     const T *G = p->tucker ? static_cast<const T *>(lam) : nullptr;
     const T *weights = p->tucker ? static_cast<const T *>(p->ones) : static_cast<const T *>(lam);
     if (p->timing) cudaEventRecord(p->ev[0], st);
+    TgAxes<T> ax;
     for (int q = 0; q < 3; ++q) {
-        tg_apply<T>(static_cast<const T *>(p->tab), p->tstride, static_cast<const T *>(U[q]), weights, p->wnode, p->R,
-                    rq[q], q, n[q], static_cast<T *>(out[q]), st);
-        p->launches++;
+        ax.U[q] = static_cast<const T *>(U[q]);
+        ax.out[q] = static_cast<T *>(out[q]);
+        ax.n[q] = n[q];
+        ax.r[q] = rq[q];
     }
+    cudaError_t ea = tg_apply<T>(static_cast<const T *>(p->tab), p->tstride, ax, weights, p->wnode, p->R, st);
+    if (ea != cudaSuccess) return tg_fail(DEMAG_ERR_CUDA, std::string("TG factor transforms: ") + cudaGetErrorString(ea));
+    p->launches++;
     const bool mma = std::is_same<T, float>::value && p->contraction == 1;
     if (p->tucker) {
         const dim3 grid(3 * p->R, p->nz);
@@ -491,7 +559,7 @@ demag_status tg_run(demag_tg_plan *p, const void *lam, const void *Ux, const voi
     if (p->timing) cudaEventRecord(p->ev[3], st);
     if (want_field || E_dev) {
         // a grid-stride kernel: no more blocks than are resident at once
-        const int64_t nrows = (int64_t)p->ny * p->nz;
+        const int64_t nrows = (int64_t)((p->ny + kTgFieldRows - 1) / kTgFieldRows) * p->nz;  // groups of rows
         int occ = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tg_field<T>, kTgFieldThreads, 0) != cudaSuccess ||
             occ < 1)
