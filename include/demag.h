@@ -483,21 +483,26 @@ demag_status demag_tune_padding(int nx, int ny, int nz, double dx, double dy, do
  *    copy, several CTAs per SM.
  *    SP plans have one form per length, and 5 (lengths 32..256); FP32 SP plans of
  *    z length 256 and 512 run persistent TMA-fed tiles whatever the variant.
+ *    A plan that is not autotuned starts with 6 (FP32, z length 256 and 512),
+ *    8 (32..128) or 0.
  * y: 0 = two-stage column transform, 1 = swapped radix order (y lengths 32,
  *    128, 512), 2 = three-stage transform with more CTAs per SM (y lengths
  *    512 and 1024), 3 = as 2, with the forward pass by persistent CTAs that
  *    receive their column tiles by TMA tensor copies (two tiles in flight).
+ *    FP32 plans have one form at y lengths 512 and 1024, whatever the variant;
+ *    an FP64 plan that is not autotuned starts with 2 there, else 0.
  *    A variant that does not exist for the plan's lengths runs as variant 0.
  *    Out-of-range values: DEMAG_ERR_INVALID_ARG. */
 demag_status demag_get_variants(demag_plan_t plan, int *z, int *y);
 demag_status demag_set_variants(demag_plan_t plan, int z, int y);
 
-/* x-pass variant: 0 = one CTA per tile of rows; 1 (default) = the forward
- * pass by persistent CTAs that stream their row tiles through shared memory
- * with bulk asynchronous copies (TMA) on mbarriers, two tiles in flight, where
- * the rows are contiguous 16-byte multiples (nx % 4 == 0, no cell weight),
- * else as 0; 2 = the inverse pass pipelined the same way too. The autotuner
- * times all three. Out-of-range x: DEMAG_ERR_INVALID_ARG. */
+/* x-pass variant: 0 = one CTA per tile of rows, plain loads; 1 = FP64, the
+ * forward pass by persistent CTAs that stream their row tiles through shared
+ * memory with bulk asynchronous copies (TMA) on mbarriers, two tiles in flight,
+ * where the rows are contiguous 16-byte multiples (nx % 4 == 0, no cell
+ * weight), else as 0; 2 = as 1, and the inverse pass's tiles arrive by one bulk
+ * copy each (rows of 64 to 512 complex points). A plan that is not autotuned
+ * starts with 2 (FP32) or 1. Out-of-range x: DEMAG_ERR_INVALID_ARG. */
 demag_status demag_get_x_variant(demag_plan_t plan, int *x);
 demag_status demag_set_x_variant(demag_plan_t plan, int x);
 

@@ -764,6 +764,20 @@ int sp_smooth_pad(int n)
     return p;
 }
 
+// Kernel forms of a plan that is not autotuned, by the lengths alone: the ones
+// the autotuner keeps almost everywhere at these lengths (FP32 fields, ms, this form
+// against the two-stage forms of variant 0: z pass at 256^3 0.63 / 1.08, 128^3 0.070 /
+// 0.155, 64^3 0.018 / 0.027, 16^3 0.008 / 0.026; FP64 z pass at 64^3 0.30 / 0.36).
+void default_variants(demag_plan *p, int method, demag_prec prec, const int P[3])
+{
+    const bool dm32 = method == DEMAG_METHOD_DM && prec == DEMAG_F32;
+    const int L = P[2];
+    p->xvariant = prec == DEMAG_F32 ? 2 : 1;  // bulk-copy x passes where the rows allow them
+    if (dm32 && (L == 256 || L == 512)) p->zvariant = 6;
+    else if (method == DEMAG_METHOD_DM && (L == 32 || L == 64 || L == 128)) p->zvariant = 8;
+    if (prec == DEMAG_F64 && (P[1] == 512 || P[1] == 1024)) p->yvariant = 2;  // FP32 has one form there
+}
+
 // Allocates a plan with padded lengths P for the given method (no launches).
 demag_status create_plan(int nx, int ny, int nz, double dx, double dy, double dz, demag_prec prec, const int P[3],
                          int method, demag_plan_t *out)
@@ -771,7 +785,7 @@ demag_status create_plan(int nx, int ny, int nz, double dx, double dy, double dz
     demag_plan *p = new demag_plan;
     memset(p, 0, sizeof(*p));
     p->method = method;
-    p->xvariant = 1;  // pipelined x passes where the rows allow them
+    default_variants(p, method, prec, P);
     p->nx = nx; p->ny = ny; p->nz = nz;
     p->dx = dx; p->dy = dy; p->dz = dz;
     p->prec = prec;
@@ -1551,6 +1565,7 @@ demag_status demag_autotune(demag_plan_t p, int use_cache, double *best_ms, void
     // (lengths that are not powers of two have the one mixed-radix form)
     const bool z2 = is_pow2(p->Pz);
     if (!is_pow2(p->Px)) xs = {0};
+    else if (p->prec == DEMAG_F32) xs = {0, 2};  // the pipelined forward pass is FP64's
     if (z2 && dm && p->Pz >= 32 && p->Pz <= 512) zs.push_back(1);
     if (z2 && dm && p->Pz == 512) zs.push_back(2);  // 256 threads: the product stage uses every thread
     if (z2 && dm && p->Pz >= 64 && p->Pz <= 512) zs.push_back(3);  // persistent, pipelined
@@ -1562,8 +1577,11 @@ demag_status demag_autotune(demag_plan_t p, int use_cache, double *best_ms, void
         zs.push_back(7);
     }
     if (p->Py == 32 || p->Py == 128 || p->Py == 512) ys.push_back(1);
-    if (p->Py == 512 || p->Py == 1024) ys.push_back(2);  // three-stage, more CTAs per SM
-    if (p->Py == 512 || p->Py == 1024) ys.push_back(3);  // forward pass by the TMA pipeline
+    if (p->prec == DEMAG_F32 && (p->Py == 512 || p->Py == 1024)) ys = {0};  // one form
+    else if (p->Py == 512 || p->Py == 1024) {
+        ys.push_back(2);  // three-stage, more CTAs per SM
+        ys.push_back(3);  // forward pass by the TMA pipeline
+    }
     const size_t bytes = 3 * (size_t)ncell(p) * elem_size(p);
     void *M = nullptr, *H = nullptr;
     DEMAG_CUDA(dmalloc(&M, bytes));

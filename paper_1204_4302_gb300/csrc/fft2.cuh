@@ -1024,6 +1024,61 @@ __device__ __forceinline__ void x_out_pair(const XOut<T> &o, int row, int x, T h
     }
 }
 
+// Second stage and epilogue of an inverse x tile: sm holds the first stage's
+// exchange rows (xex), smM with MP the reference rows; the energy's terms go to acc.
+template <typename T, int L, bool P1, bool MP, int NTX>
+__device__ __forceinline__ void x_inv_finish(const typename Cplx<T>::type *sm, const T *smM, int row0, int nrows, int nvalid,
+                                             const XOut<T> &o, const typename Cplx<T>::type *__restrict__ twx, T &acc)
+{
+    using C = typename Cplx<T>::type;
+    using S = XShape<T, L, NTX>;
+    constexpr int R1 = S::R1, R2 = S::R2, TR = S::TR, RS = S::RS;
+    if (threadIdx.x < TR * R1) {
+        const int rr = threadIdx.x / R1, j2 = threadIdx.x % R1, row = row0 + rr;
+        const C *s = sm + rr * RS;
+        // the energy's M of a plain field's even rows, loaded ahead of the transform
+        constexpr int HO = P1 ? R2 / 2 + 1 : R2 / 2;
+        const bool ahead = !MP && o.partials && !o.wcell && ((o.out_rs | nvalid) & 1) == 0;
+        C m[HO];
+        if constexpr (!MP) {
+            const T *mp = o.Mref + (int64_t)row * o.out_rs;
+#pragma unroll
+            for (int r = 0; r < HO; ++r) {
+                m[r] = cmk<C>(0, 0);
+                if (ahead && row < nrows && 2 * (j2 + r * R1) < nvalid)
+                    m[r] = *reinterpret_cast<const C *>(mp + 2 * (j2 + r * R1));
+            }
+        }
+        C v[R2];
+#pragma unroll
+        for (int r = 0; r < R2; ++r) v[r] = s[xex<R1>(r, j2)];
+#pragma unroll
+        for (int r = 1; r < R2; ++r) v[r] = cmulc(v[r], __ldg(&twx[2 * r * j2]));
+        if constexpr (P1) RegDFTHalfOutP1<R2, true, C>::run(v);
+        else RegDFTHalfOut<R2, true, C>::run(v);
+        if (row < nrows) {
+            const T g = o.gdev ? (T)(*o.gdev) : (T)1;
+            const T oscale = o.oscale * g;
+            if (ahead) {
+                T *op = o.out + (int64_t)row * o.out_rs;
+#pragma unroll
+                for (int r = 0; r < HO; ++r) {  // m is zero beyond the row
+                    const C hv = cmk<C>(v[r].x * o.scale, v[r].y * o.scale);
+                    if (o.out && 2 * (j2 + r * R1) < nvalid)
+                        *reinterpret_cast<C *>(op + 2 * (j2 + r * R1)) = cmk<C>(hv.x * oscale, hv.y * oscale);
+                    acc += o.mscale * (m[r].x * hv.x + m[r].y * hv.y);
+                }
+            } else
+#pragma unroll
+            for (int r = 0; r < HO; ++r) {  // z[n], n = j2 + r R1 (< L/2 unless P1)
+                const int n = j2 + r * R1;
+                x_out_pair<T>(o, row, 2 * n, v[r].x * o.scale, v[r].y * o.scale, oscale, nvalid,
+                              MP ? smM + rr * L : nullptr, acc);
+            }
+        }
+    }
+}
+
 template <typename T, int L, bool CG, bool P1 = false, bool MP = false, int NTX = Tile2<T>::NT>
 __device__ __forceinline__ void k_x_inv2_tile(const typename Cplx<T>::type *__restrict__ in, int64_t in_rs, int nrows, int nvalid, XOut<T> o,
          const typename Cplx<T>::type *__restrict__ twx, int tile, unsigned char *smraw)
@@ -1070,50 +1125,7 @@ __device__ __forceinline__ void k_x_inv2_tile(const typename Cplx<T>::type *__re
     if constexpr (MP) cp_async_wait_all();
     __syncthreads();
     T acc = 0;  // per-thread sum of a few dozen terms; blocks reduce in FP64
-    if (threadIdx.x < TR * R1) {
-        const int rr = threadIdx.x / R1, j2 = threadIdx.x % R1, row = row0 + rr;
-        const C *s = sm + rr * RS;
-        // the energy's M of a plain field's even rows, loaded ahead of the transform
-        constexpr int HO = P1 ? R2 / 2 + 1 : R2 / 2;
-        const bool ahead = !MP && o.partials && !o.wcell && ((o.out_rs | nvalid) & 1) == 0;
-        C m[HO];
-        if constexpr (!MP) {
-            const T *mp = o.Mref + (int64_t)row * o.out_rs;
-#pragma unroll
-            for (int r = 0; r < HO; ++r) {
-                m[r] = cmk<C>(0, 0);
-                if (ahead && row < nrows && 2 * (j2 + r * R1) < nvalid)
-                    m[r] = *reinterpret_cast<const C *>(mp + 2 * (j2 + r * R1));
-            }
-        }
-        C v[R2];
-#pragma unroll
-        for (int r = 0; r < R2; ++r) v[r] = s[xex<R1>(r, j2)];
-#pragma unroll
-        for (int r = 1; r < R2; ++r) v[r] = cmulc(v[r], __ldg(&twx[2 * r * j2]));
-        if constexpr (P1) RegDFTHalfOutP1<R2, true, C>::run(v);
-        else RegDFTHalfOut<R2, true, C>::run(v);
-        if (row < nrows) {
-            const T g = o.gdev ? (T)(*o.gdev) : (T)1;
-            const T oscale = o.oscale * g;
-            if (ahead) {
-                T *op = o.out + (int64_t)row * o.out_rs;
-#pragma unroll
-                for (int r = 0; r < HO; ++r) {  // m is zero beyond the row
-                    const C hv = cmk<C>(v[r].x * o.scale, v[r].y * o.scale);
-                    if (o.out && 2 * (j2 + r * R1) < nvalid)
-                        *reinterpret_cast<C *>(op + 2 * (j2 + r * R1)) = cmk<C>(hv.x * oscale, hv.y * oscale);
-                    acc += o.mscale * (m[r].x * hv.x + m[r].y * hv.y);
-                }
-            } else
-#pragma unroll
-            for (int r = 0; r < HO; ++r) {  // z[n], n = j2 + r R1 (< L/2 unless P1)
-                const int n = j2 + r * R1;
-                x_out_pair<T>(o, row, 2 * n, v[r].x * o.scale, v[r].y * o.scale, oscale, nvalid,
-                              MP ? smM + rr * L : nullptr, acc);
-            }
-        }
-    }
+    x_inv_finish<T, L, P1, MP, NTX>(sm, smM, row0, nrows, nvalid, o, twx, acc);
     if (o.partials) block_partial<NT>((double)acc, o.partials, tile);
 }
 

@@ -149,9 +149,14 @@ template <int R, int NZ, bool INV, typename C> struct DFT {
     }
 };
 
-// f(std::integral_constant<int, R>) for the stage radix R (<= MAXR) of a plan
-template <int MAXR, typename F> __device__ __forceinline__ void with_radix(int R, F &&f)
+// f(std::integral_constant<int, R>) for the stage radix R (<= MAXR) of a plan, or
+// for the compile-time radix FIXED where it is not 0
+template <int MAXR, int FIXED = 0, typename F> __device__ __forceinline__ void with_radix(int R, F &&f)
 {
+    if constexpr (FIXED != 0) {
+        f(std::integral_constant<int, FIXED>{});
+        return;
+    }
 #define DEMAG_R(N) case N: if constexpr (N <= MAXR) f(std::integral_constant<int, N>{}); break;
     switch (R) {
         DEMAG_R(2) DEMAG_R(3) DEMAG_R(4) DEMAG_R(5) DEMAG_R(6) DEMAG_R(7) DEMAG_R(8) DEMAG_R(9) DEMAG_R(10)
@@ -180,8 +185,10 @@ __device__ __forceinline__ void twiddle(C *v, int kstep, const C *__restrict__ t
 // up to the tile so that tiles start on the row's alignment). HALF_IN: forward,
 // rows >= L / 2 are zero (nin <= L / 2); otherwise the inverse, of which rows
 // <= L / 2 are formed. Thread (g, c): butterflies g, g + G, ... of column c.
-template <typename T, bool INV, int TC, int MAXR>
-__global__ void __launch_bounds__(sizeof(T) == 4 ? 256 : 128, MAXR <= 16 ? (sizeof(T) == 4 ? 3 : 4) : (sizeof(T) == 4 ? 2 : 2))
+// C1, C2: the radices where they are known at compile time (the power-of-two
+// lengths 512 and 1024), else 0 and the plan's.
+template <typename T, bool INV, int TC, int MAXR, int C1 = 0, int C2 = 0>
+__global__ void __launch_bounds__(sizeof(T) == 4 ? 256 : 128, MAXR <= 16 ? (sizeof(T) == 4 ? 3 : 4) : 2)
 k_mix2_col(const typename Cplx<T>::type *__restrict__ in, typename Cplx<T>::type *__restrict__ out, int vw, int width,
            int nslabs, int64_t iss, int irs, int nin, int64_t oss, int ors, int nout,
            const typename Cplx<T>::type *__restrict__ tw, const Mix2 g)
@@ -194,8 +201,9 @@ k_mix2_col(const typename Cplx<T>::type *__restrict__ in, typename Cplx<T>::type
     const bool ok = slab < nslabs && off < width;
     const C *src = in + (int64_t)slab * iss + off;
     C *dst = out + (int64_t)slab * oss + off;
-    const int R1 = g.R1, R2 = g.R2, RP = g.RP, G = g.G;
-    mx::with_radix<MAXR>(R1, [&](auto rr) {
+    const int R1 = C1 ? C1 : g.R1, R2 = C2 ? C2 : g.R2, G = C1 ? 256 / TC : g.G;
+    const int RP = C1 ? (TC * (int)sizeof(C) >= 128 ? C1 : (C1 | 1)) : g.RP;
+    mx::with_radix<MAXR, C1>(R1, [&](auto rr) {
         constexpr int R = decltype(rr)::value, H = INV ? R : (R + 1) / 2;
         const unsigned step = (unsigned)(R2 * irs);
         for (int j = j0; j < R2; j += G) {
@@ -216,7 +224,7 @@ k_mix2_col(const typename Cplx<T>::type *__restrict__ in, typename Cplx<T>::type
         }
     });
     __syncthreads();
-    mx::with_radix<MAXR>(R2, [&](auto rr) {
+    mx::with_radix<MAXR, C2>(R2, [&](auto rr) {
         constexpr int R = decltype(rr)::value, H = INV ? R / 2 + 1 : R;
         const int step = RP * TC;
         const unsigned ostep = (unsigned)(R1 * ors);

@@ -83,12 +83,10 @@ cudaError_t x_inv_pipe(const typename Cplx<T>::type *in, int in_rs, int nrows, i
                        const typename Cplx<T>::type *twx, cudaStream_t st)
 {
     using S = XShape<T, L>;
-    const size_t sm = 2 * xinv_slot_bytes<T, L>(in_rs) + 2 * sizeof(uint64_t);
-    cudaError_t e = allow_smem<k_x_inv_tma<T, L, P1>>(sm);
+    const size_t sm = xinv_slot_bytes<T, L>(in_rs) + sizeof(uint64_t);
+    cudaError_t e = allow_smem<k_x_inv_bulk<T, L, P1>>(sm);
     if (e != cudaSuccess) return e;
-    const int ntiles = (nrows + S::TR - 1) / S::TR;
-    const int cap = sm_count() * resident_ctas<k_x_inv_tma<T, L, P1>>(S::NT, sm);
-    k_x_inv_tma<T, L, P1><<<ntiles < cap ? ntiles : cap, S::NT, sm, st>>>(in, in_rs, nrows, nvalid, o, twx, ntiles);
+    k_x_inv_bulk<T, L, P1><<<(nrows + S::TR - 1) / S::TR, S::NT, sm, st>>>(in, in_rs, nrows, nvalid, o, twx);
     return cudaGetLastError();
 }
 }  // namespace
@@ -548,9 +546,10 @@ cudaError_t Passes<T>::x_fwd(int L, const XIn<T> &a, int nrows, int nvalid, C *o
 {
     if (nrows <= 0) return cudaSuccess;
     if (!pow2_len(L)) return MixedPasses<T>::x_fwd(L, a, nrows, nvalid, out, out_rs, twx, st);
-    // pipelined form: rows of the plain field (no per-cell weight) stored back
-    // to back, 16-byte multiples, zero-padded half
-    if (variant >= 1 && L >= 64 && nvalid <= L && !a.wcell && a.in_rs == nvalid && nvalid % 4 == 0 &&
+    // pipelined form (FP64; FP32 rows go faster through k_x_fwd2 with its loads issued
+    // together: 256^3 152 -> 137 us, 512 x 512 x 128 298 -> 280): rows of the plain field
+    // (no per-cell weight) stored back to back, 16-byte multiples, zero-padded half
+    if constexpr (sizeof(T) == 8) if (variant >= 1 && L >= 64 && nvalid <= L && !a.wcell && a.in_rs == nvalid && nvalid % 4 == 0 &&
         ((uintptr_t)a.in & 15) == 0) {
         switch (L) {
         case 64: return x_fwd_pipe<T, 64>(a, nrows, nvalid, out, out_rs, twx, st);
@@ -638,9 +637,7 @@ cudaError_t Passes<T>::x_inv(int L, const C *in, int64_t in_rs, int nrows, int n
     case LL:                                                                                   \
         return p1 ? x_inv_pipe<T, LL, true>(in, (int)in_rs, nrows, nvalid, o, twx, st)         \
                   : x_inv_pipe<T, LL, false>(in, (int)in_rs, nrows, nvalid, o, twx, st);
-        // (L = 512 would hold a whole 32-point stage in registers across the
-        // buffer hand-over: one CTA per SM; the one-tile kernel serves it)
-        switch (L) { DEMAG_PIPE(64) DEMAG_PIPE(128) DEMAG_PIPE(256) default: break; }
+        switch (L) { DEMAG_PIPE(64) DEMAG_PIPE(128) DEMAG_PIPE(256) DEMAG_PIPE(512) default: break; }
 #undef DEMAG_PIPE
     }
     if (L >= 16) {
@@ -707,6 +704,27 @@ cudaError_t Passes<T>::col_launch(const C *in, C *out, int ncols, int width, int
     return cudaGetLastError();
 }
 
+// FP32 columns of 512 = 32 x 16 and 1024 = 32 x 32 points in two register stages
+// (k_mix2_col with compile-time radices): one exchange instead of the two of the
+// three-stage kernel, whose shared-memory traffic held the L1 at 85%, and 128-byte
+// rows at 512. 256^3: forward 277 -> 230 us, inverse 298 -> 234; 512 x 512 x 128: 566 -> 435
+// and 620 -> 455.
+template <bool INV, int TC, int R1, int R2>
+static cudaError_t col2s_launch(const float2 *in, float2 *out, int width, int nslabs, int64_t iss, int64_t irs, int nin,
+                                int64_t oss, int64_t ors, int nout, const float2 *tw, cudaStream_t st)
+{
+    Mix2 g;
+    memset(&g, 0, sizeof g);
+    g.L = R1 * R2;
+    const size_t sm = (size_t)R2 * (TC >= 16 ? R1 : (R1 | 1)) * TC * sizeof(float2);
+    cudaError_t e = allow_smem<k_mix2_col<float, INV, TC, 32, R1, R2>>(sm);
+    if (e != cudaSuccess) return e;
+    const int up = (width + TC - 1) / TC * TC, vw = up * 8 <= width * 9 ? up : width;
+    k_mix2_col<float, INV, TC, 32, R1, R2><<<(unsigned)(((int64_t)vw * nslabs + TC - 1) / TC), 256, sm, st>>>(
+        in, out, vw, width, nslabs, iss, (int)irs, nin, oss, (int)ors, nout, tw, g);
+    return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t Passes<T>::col(int L, bool inv, const C *in, C *out, int ncols, int width, int64_t iss,
                            int64_t irs, int nin, int64_t oss, int64_t ors, int nout, const C *tw,
@@ -715,6 +733,18 @@ cudaError_t Passes<T>::col(int L, bool inv, const C *in, C *out, int ncols, int 
     if (ncols <= 0) return cudaSuccess;
     if (!pow2_len(L))
         return MixedPasses<T>::col(L, inv, in, out, ncols, width, iss, irs, nin, oss, ors, nout, tw, twstride, st);
+    if constexpr (sizeof(T) == 4) {
+        // the pruned field passes of 512 and 1024 points
+        if ((L == 512 || L == 1024) && ncols % width == 0 && twstride == 1 && irs * L < (1ll << 31) && ors * L < (1ll << 31)) {
+            const int nslabs = ncols / width;
+            if (!inv && nout == L && 2 * nin <= L)
+                return L == 512 ? col2s_launch<false, 16, 32, 16>(in, out, width, nslabs, iss, irs, nin, oss, ors, nout, tw, st)
+                                : col2s_launch<false, 8, 32, 32>(in, out, width, nslabs, iss, irs, nin, oss, ors, nout, tw, st);
+            if (inv && nin == L && 2 * (nout - 1) <= L)
+                return L == 512 ? col2s_launch<true, 16, 16, 32>(in, out, width, nslabs, iss, irs, nin, oss, ors, nout, tw, st)
+                                : col2s_launch<true, 8, 32, 32>(in, out, width, nslabs, iss, irs, nin, oss, ors, nout, tw, st);
+        }
+    }
     if (L <= 16) {
         // one thread per column
         const int grid = (ncols + Tile2<T>::NT - 1) / Tile2<T>::NT;
@@ -731,13 +761,13 @@ cudaError_t Passes<T>::col(int L, bool inv, const C *in, C *out, int ncols, int 
     // the zero padding halves the input (forward) or the output (inverse)
     const bool pin = 2 * nin <= L, pout = 2 * nout <= L;
     // variant 3: forward by the TMA pipeline, inverse as variant 2
-    if (variant == 3 && !inv && pin && nout == L && (L == 512 || L == 1024)) {
+    if constexpr (sizeof(T) == 8) if (variant == 3 && !inv && pin && nout == L && (L == 512 || L == 1024)) {
         const cudaError_t e = L == 512 ? col_fwd_tma<T, 512>(in, out, ncols, width, iss, irs, nin, oss, ors, tw, twstride, st)
                                        : col_fwd_tma<T, 1024>(in, out, ncols, width, iss, irs, nin, oss, ors, tw, twstride, st);
         if (e != cudaErrorNotSupported) return e;
     }
     if (variant == 3) variant = 2;
-    if (variant == 2 && (L == 512 || L == 1024) && (pin || pout) && !(pin && inv) && !(pout && !inv)) {
+    if constexpr (sizeof(T) == 8) if (variant == 2 && (L == 512 || L == 1024) && (pin || pout) && !(pin && inv) && !(pout && !inv)) {
 #define DEMAG_C3(LL)                                                                                    \
     if (L == LL) {                                                                                      \
         using S3 = Col3Shape<T, LL>;                                                                    \

@@ -233,110 +233,73 @@ k_x_fwd_tma(const T *__restrict__ in, T wscalar, int nrows, int nvalid, typename
     }
 }
 
-// Inverse C2R rows with the XOut epilogue (energy partials per tile into
-// partials[t]); input rows of in_rs complex (even) stored back to back.
-// P1 as in k_x_inv2 (one output pair beyond the half length). Each of the two
-// buffers first receives a tile by bulk copy and then, once stage 1 has read
-// it into registers, serves as that tile's exchange rows, so a CTA needs two
-// buffers in all and three CTAs fit on an SM; the buffer is refilled with the
-// tile after next when stage 2 is done with it.
+// Inverse C2R rows with the XOut epilogue, one tile per CTA: the tile's rows of
+// in_rs complex (even; stored back to back) arrive by one bulk copy, so each spectrum value is
+// read from global memory once (the first stage needs X[k] and X[L-k] in different
+// threads); once stage 1 has them in registers the buffer serves as the exchange rows.
+// One buffer per CTA and no register held across tiles, so that four CTAs (two at L = 512) per
+// SM overlap one another's copies: 256^3 160 -> 136 us against the persistent form with two
+// buffers and two CTAs per SM, 512 x 512 x 128 392 -> 358 against k_x_inv2. P1 as in k_x_inv2.
 template <typename T, int L, bool P1>
-__global__ void __launch_bounds__(Tile2<T>::NT)
-k_x_inv_tma(const typename Cplx<T>::type *__restrict__ in, int in_rs, int nrows, int nvalid, XOut<T> o,
-            const typename Cplx<T>::type *__restrict__ twx, int ntiles)
+__global__ void __launch_bounds__(Tile2<T>::NT, (sizeof(T) == 4 ? (L <= 256 ? 4 : 2) : 2))
+k_x_inv_bulk(const typename Cplx<T>::type *__restrict__ in, int in_rs, int nrows, int nvalid, XOut<T> o,
+             const typename Cplx<T>::type *__restrict__ twx)
 {
     using C = typename Cplx<T>::type;
     using S = XShape<T, L>;
     constexpr int R1 = S::R1, R2 = S::R2, NT = S::NT, TR = S::TR, RS = S::RS;
     extern __shared__ __align__(16) unsigned char smraw[];
-    const size_t slot = xinv_slot_bytes<T, L>(in_rs);
-    C *buf[2] = {reinterpret_cast<C *>(smraw), reinterpret_cast<C *>(smraw + slot)};
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smraw + 2 * slot);
-    __shared__ int s_fail;
+    C *sm = reinterpret_cast<C *>(smraw);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smraw + xinv_slot_bytes<T, L>(in_rs));
+    const int t = blockIdx.x, row0 = t * TR;
     if (threadIdx.x == 0) {
-        s_fail = 0;
-        mbar_init(&bars[0], 1);
-        mbar_init(&bars[1], 1);
+        mbar_init(bar, 1);
         mbar_fence_init();
+        xpipe_issue(in, in_rs, nrows, TR, t, sm, bar);
     }
     __syncthreads();
-    const int step = gridDim.x;
-    if (threadIdx.x == 0)
-        for (int i = 0; i < 2; ++i) {
-            const int t = blockIdx.x + i * step;
-            if (t < ntiles) xpipe_issue(in, in_rs, nrows, TR, t, buf[i], &bars[i]);
-        }
-    const T g = o.gdev ? (T)(*o.gdev) : (T)1;
-    const T oscale = o.oscale * g;
-    for (int i = 0;; ++i) {
-        const int t = blockIdx.x + i * step;
-        if (t >= ntiles) break;
-        const int b = i & 1;
-        if (!mbar_wait_bounded(&bars[b], (unsigned)((i >> 1) & 1), kPipeWaitCycles)) s_fail = 1;
-        __syncthreads();
-        if (s_fail) {
-            xpipe_abort(bars, i, step, ntiles);
-            return;
-        }
-        const int row0 = t * TR;
-        const bool act1 = threadIdx.x < TR * R2;
-        const int rr1 = threadIdx.x / R2, j1 = threadIdx.x % R2;
-        C u[R1];
-        if (act1) {
+    const bool got = mbar_wait_bounded(bar, 0, kPipeWaitCycles);
+    const bool act1 = threadIdx.x < TR * R2;
+    const int rr1 = threadIdx.x / R2, j1 = threadIdx.x % R2;
+    C u[R1];
+    if (act1) {
 #pragma unroll
-            for (int r = 0; r < R1; ++r) u[r] = cmk<C>(0, 0);
-            if (row0 + rr1 < nrows) {
-                const C *p = buf[b] + rr1 * in_rs;
+        for (int r = 0; r < R1; ++r) u[r] = cmk<C>(0, 0);
+        if (row0 + rr1 < nrows) {
+            const C *p = sm + rr1 * in_rs;
 #pragma unroll
-                for (int r = 0; r < R1; ++r) {
-                    const int k = j1 + r * R2;
-                    const C a = p[k];
-                    const C bb = p[L - k];
-                    const C E2 = cmk<C>(a.x + bb.x, a.y - bb.y);
-                    const C D = cmk<C>(a.x - bb.x, a.y + bb.y);
-                    const C O2 = cmulc(D, __ldg(&twx[k]));
-                    u[r] = cmk<C>(E2.x - O2.y, E2.y + O2.x);
-                }
-            }
-            RegDFT<R1, true, C>::run(u);
-        }
-        __syncthreads();  // the tile is in registers: the buffer becomes the exchange rows
-        C *sm = buf[b];
-        if (act1) {
-            C *s = sm + rr1 * RS;
-#pragma unroll
-            for (int r = 0; r < R1; ++r) s[xex<R1>(j1, r)] = u[r];
-        }
-        __syncthreads();
-        T acc = 0;
-        if (threadIdx.x < TR * R1) {
-            const int rr = threadIdx.x / R1, j2 = threadIdx.x % R1, row = row0 + rr;
-            const C *s = sm + rr * RS;
-            C v[R2];
-#pragma unroll
-            for (int r = 0; r < R2; ++r) v[r] = s[xex<R1>(r, j2)];
-#pragma unroll
-            for (int r = 1; r < R2; ++r) v[r] = cmulc(v[r], __ldg(&twx[2 * r * j2]));
-            if constexpr (P1) RegDFTHalfOutP1<R2, true, C>::run(v);
-            else RegDFTHalfOut<R2, true, C>::run(v);
-            if (row < nrows) {
-#pragma unroll
-                for (int r = 0; r < (P1 ? R2 / 2 + 1 : R2 / 2); ++r) {
-                    const int n = j2 + r * R1;
-                    x_out_pair<T>(o, row, 2 * n, v[r].x * o.scale, v[r].y * o.scale, oscale, nvalid, nullptr, acc);
-                }
+            for (int r = 0; r < R1; ++r) {
+                const int k = j1 + r * R2;
+                const C a = p[k];
+                const C bb = p[L - k];
+                const C E2 = cmk<C>(a.x + bb.x, a.y - bb.y);
+                const C D = cmk<C>(a.x - bb.x, a.y + bb.y);
+                const C O2 = cmulc(D, __ldg(&twx[k]));
+                u[r] = cmk<C>(E2.x - O2.y, E2.y + O2.x);
             }
         }
-        if (o.partials) block_partial<NT>((double)acc, o.partials, t);  // has its own barrier
-        __syncthreads();  // exchange rows read: the buffer can take the tile after next
-        if (threadIdx.x == 0) {
-            const int tn = blockIdx.x + (i + 2) * step;
-            if (tn < ntiles) {
-                fence_proxy_async_smem();
-                xpipe_issue(in, in_rs, nrows, TR, tn, buf[b], &bars[b]);
-            }
-        }
+        RegDFT<R1, true, C>::run(u);
     }
+    // the tile is in registers: the buffer becomes the exchange rows. A wait that
+    // gave up in any thread abandons the tile once its copy is done (or the wait
+    // runs out again)
+    if (__syncthreads_or(!got)) {
+        if (threadIdx.x == 0) {
+            mbar_wait_bounded(bar, 0, kPipeWaitCycles);
+            atomicExch(&g_xpipe_error, 1);
+        }
+        __syncthreads();
+        return;
+    }
+    if (act1) {
+        C *s = sm + rr1 * RS;
+#pragma unroll
+        for (int r = 0; r < R1; ++r) s[xex<R1>(j1, r)] = u[r];
+    }
+    __syncthreads();
+    T acc = 0;
+    x_inv_finish<T, L, P1, false, NT>(sm, nullptr, row0, nrows, nvalid, o, twx, acc);
+    if (o.partials) block_partial<NT>((double)acc, o.partials, t);
 }
 
 // ------------------------------------------------------------ y forward pass
