@@ -423,13 +423,16 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_energy_finalize(const doub
 #pragma unroll
         for (int w = 1; w < NW; ++w) two_sum_add(s, c, ss[lane + 32 * w], sc[lane + 32 * w]);
         warp_two_sum(s, c);
-        if (lane == 0) {
+        if (nb == 1) {
+            if (lane == 0) *E = factor * (s + c);
+        } else if (lane == 0) {
             scratch[2 * blockIdx.x] = s;
             scratch[2 * blockIdx.x + 1] = c;
             __threadfence();
             s_last = atomicAdd(count, 1u) == (unsigned)(nb - 1);
         }
     }
+    if (nb == 1) return;
     __syncthreads();
     if (s_last && warp == 0) {
         __threadfence();
@@ -714,7 +717,9 @@ cudaError_t sp_extract(const double2 *S, int comp, int Px, int Py, int Pz, int K
 
 cudaError_t energy_finalize(const double *partials, int n, double factor, double *E, double *scratch, cudaStream_t st)
 {
-    const int nb = std::max(1, std::min(kFinalizeBlocks, (n + 127) / 128));
+    // up to 512 partials in one CTA: three more adds per thread cost less than a second
+    // round through memory
+    const int nb = n <= 512 ? 1 : std::min(kFinalizeBlocks, (n + 127) / 128);
     k_energy_finalize<<<nb, kFinalizeThreads, 0, st>>>(partials, n, factor, E, scratch);
     return cudaGetLastError();
 }
