@@ -110,6 +110,7 @@ k_tg_apply(const T *__restrict__ tab, int tstride, const T *__restrict__ lam, co
     T *__restrict__ out = ax.out[q];
     T *su = reinterpret_cast<T *>(smraw);   // [n][VC]
     T *st = su + (size_t)n * VC;             // [2n - 1]
+    __shared__ T scale[VC];
     const int lp = blockIdx.x;               // l * 3 + p
     const int p = lp % 3, l = lp / 3;
     const T *tb = tab + ((int64_t)(l * 3 + q) * 2 + (p == q ? 1 : 0)) * tstride;
@@ -121,6 +122,10 @@ k_tg_apply(const T *__restrict__ tab, int tstride, const T *__restrict__ lam, co
             const int mm = e / n, j = e - mm * n;
             su[j * VC + mm] = mm < mc ? U[((int64_t)p * r + m0 + mm) * n + j] : (T)0;
         }
+        if ((int)threadIdx.x < mc)
+            scale[threadIdx.x] = q == 0 ? (T)(wnode[l] * (double)lam[p * r + m0 + threadIdx.x] *
+                                              (1.0 / (4.0 * 3.14159265358979323846)))
+                                        : (T)1;
         __syncthreads();
         for (int i0 = threadIdx.x; i0 < n; i0 += kTgNO * blockDim.x) {
             T acc[kTgNO][VC];
@@ -152,10 +157,7 @@ k_tg_apply(const T *__restrict__ tab, int tstride, const T *__restrict__ lam, co
                 const int i = i0 + o * (int)blockDim.x;
                 if (i >= n) continue;
                 for (int mm = 0; mm < mc; ++mm) {
-                    const int m = m0 + mm, v = lp * r + m;
-                    T scale = (T)1;
-                    if (q == 0) scale = (T)(wnode[l] * (double)lam[p * r + m] * (1.0 / (4.0 * 3.14159265358979323846)));
-                    out[(int64_t)v * n + i] = acc[o][mm] * scale;
+                    out[((int64_t)lp * r + m0 + mm) * n + i] = acc[o][mm] * scale[mm];
                 }
             }
         }
@@ -372,7 +374,7 @@ k_tg_field(const T *__restrict__ phi, int nx, int ny, int nz, T hx, T hy, T hz, 
 // (the core times the transformed y and z factors). One block per ((l,p), k):
 // U[a][b] = sum_c G[c][b][a] Z[(l,p,c)][k] in shared memory, then
 // Q = sum_b U[a][b] Y[(l,p,b)][j] over the block's threads. KMAJOR: Q stored
-// [g][Kp] (rows of the tensor-core operand), else [K][g] (the CUDA-core form).
+// in the order of tgm::kpos (the tensor-core operand), else [K][g] (the CUDA-core form).
 template <typename T, bool KMAJOR>
 __global__ void __launch_bounds__(256)
 k_tg_tucker_q(const T *__restrict__ G, const T *__restrict__ Y, const T *__restrict__ Z, int r1, int r2, int r3,
@@ -394,7 +396,7 @@ k_tg_tucker_q(const T *__restrict__ G, const T *__restrict__ Y, const T *__restr
         T acc = 0;
         for (int b = 0; b < r2; ++b) acc += U[a * r2 + b] * Y[((int64_t)lp * r2 + b) * ny + j];
         const int64_t g = (int64_t)k * ny + j, K = (int64_t)lp * r1 + a;
-        if (KMAJOR) Q[g * Kp + K] = acc;
+        if (KMAJOR) Q[tgm::kpos(K, g, M)] = acc;
         else Q[K * M + g] = acc;
     }
     if (KMAJOR && lp == (int)gridDim.x - 1) {
@@ -402,7 +404,7 @@ k_tg_tucker_q(const T *__restrict__ G, const T *__restrict__ Y, const T *__restr
         // and term-major forms share the buffer)
         const int K = (int)gridDim.x * r1, pad = Kp - K;
         for (int e = threadIdx.x; e < ny * pad; e += blockDim.x)
-            Q[((int64_t)k * ny + e / pad) * Kp + K + e % pad] = (T)0;
+            Q[tgm::kpos(K + e % pad, (int64_t)k * ny + e / pad, M)] = (T)0;
     }
 }
 
@@ -452,7 +454,7 @@ demag_status tg_fail(demag_status s, const std::string &m)
 }
 
 // The FP32 contraction on the tensor cores: operand preparation (B in stage
-// order with its TF32 split, Y and Z transposed to K-contiguous rows), then
+// order with its TF32 split, Y and Z transposed to the order of kpos), then
 // the persistent tcgen05 kernel.
 // Tucker plans pass their operand Q [nz ny][Kp] as the y factor of ny_eff =
 // nz ny rows and a row of ones as the z factor (nz_eff = 1): A = Q * 1.
@@ -472,9 +474,9 @@ cudaError_t tg_contract_mma(demag_tg_plan *p, float *phi, cudaStream_t st, cudaE
         ny = p->ny * p->nz;
         nz = 1;
     } else {
-        const int by = (int)std::min<int64_t>(((int64_t)p->ny * p->Kp + 255) / 256, 4096);
+        const int by = (int)std::min<int64_t>(((int64_t)p->ny * p->Kp / 8 + 255) / 256, 4096);
         tgm::k_tg_transpose<<<by, 256, 0, st>>>(static_cast<const float *>(p->Y), K, p->ny, p->Kp, p->Yt);
-        const int bz = (int)std::min<int64_t>(((int64_t)p->nz * p->Kp + 255) / 256, 4096);
+        const int bz = (int)std::min<int64_t>(((int64_t)p->nz * p->Kp / 8 + 255) / 256, 4096);
         tgm::k_tg_transpose<<<bz, 256, 0, st>>>(static_cast<const float *>(p->Z), K, p->nz, p->Kp, p->Zt);
         p->launches += 2;
     }

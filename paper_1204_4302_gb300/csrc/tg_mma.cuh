@@ -23,7 +23,7 @@
 //     N BN, K 8 per instruction; 6 per stage) and commits them to the
 //     stage's "empty" barrier and, after a tile, to "tile full";
 //   warps 2..9: form A = Z Y for 128 rows x 16 K per stage from the
-//     transposed factors (two threads per row, 8 K each), split it into hi
+//     transposed factors (order of kpos; two threads per row, 8 K each), split it into hi
 //     and lo and store them in the 64-byte-swizzled K-major layout; after a
 //     tile, read both accumulators back (tcgen05.ld; warp w reads TMEM lanes
 //     32 (w mod 4) .., warps 2..5 and 6..9 alternate 32-column chunks), add
@@ -250,14 +250,24 @@ __global__ void k_tg_prep_b(const float *__restrict__ X, int K, int nx, int BN, 
     }
 }
 
-// F[K][n] -> Ft[n][Kp] (zero for K >= the term count).
+// Position of term K of row j (n rows) in the transposed factors: eight terms of a
+// row together, the rows of such a group side by side. A producer thread's eight
+// terms of a stage are then 32 bytes next to its neighbour's, eight lines per warp load
+// instead of the 32 of K-contiguous rows, which held the L1 at 72%.
+__host__ __device__ __forceinline__ int64_t kpos(int64_t K, int64_t j, int64_t n) { return ((K >> 3) * n + j) * 8 + (K & 7); }
+
+// F[K][n] -> Ft in the order of kpos (zero for K >= the term count), K < Kp.
 __global__ void k_tg_transpose(const float *__restrict__ F, int K, int n, int Kp, float *__restrict__ Ft)
 {
-    const int64_t total = (int64_t)n * Kp;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int Kk = (int)(e % Kp), j = (int)(e / Kp);
-        Ft[e] = Kk < K ? F[(int64_t)Kk * n + j] : 0.0f;
+    const int total = n * (Kp / 8);
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+        const int kg = e / n, j = e - kg * n;
+        float v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = kg * 8 + q < K ? F[(int64_t)(kg * 8 + q) * n + j] : 0.0f;
+        float4 *dst = reinterpret_cast<float4 *>(Ft + (int64_t)e * 8);
+        dst[0] = make_float4(v[0], v[1], v[2], v[3]);
+        dst[1] = make_float4(v[4], v[5], v[6], v[7]);
     }
 }
 
@@ -363,17 +373,25 @@ k_tg_mma(const float *__restrict__ Yt, const float *__restrict__ Zt, const float
             const int g = mt * kBM + m;
             const bool valid = g < M;
             const int k = valid ? g / ny : 0, j = valid ? g % ny : 0;
-            const float4 *yrow = reinterpret_cast<const float4 *>(Yt + (int64_t)j * Kp) + 2 * kh;
-            const float4 *zrow = reinterpret_cast<const float4 *>(Zt + (int64_t)k * Kp) + 2 * kh;
+            const float4 *yrow = reinterpret_cast<const float4 *>(Yt + kpos(8 * kh, j, ny));
+            const float4 *zrow = reinterpret_cast<const float4 *>(Zt + kpos(8 * kh, k, nz));
             bool ok = true;
-            for (int kc = 0; kc < nkc; ++kc, ++it) {
-                const int s = it % kStages;
-                float4 y[2], z[2];
+            // the factors are loaded one stage ahead: a stage needs all eight
+            // producer warps, and with the loads' latency in every stage they, not the tensor
+            // pipe, set its time
+            float4 yn[2], zn[2];
+            auto load = [&](int kc) {
 #pragma unroll
                 for (int c = 0; c < 2; ++c) {
-                    y[c] = valid ? __ldg(yrow + kc * 4 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    z[c] = valid ? __ldg(zrow + kc * 4 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    yn[c] = valid ? __ldg(yrow + (int64_t)kc * 4 * ny + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    zn[c] = valid ? __ldg(zrow + (int64_t)kc * 4 * nz + c) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
+            };
+            load(0);
+            for (int kc = 0; kc < nkc; ++kc, ++it) {
+                const int s = it % kStages;
+                const float4 y[2] = {yn[0], yn[1]}, z[2] = {zn[0], zn[1]};
+                if (kc + 1 < nkc) load(kc + 1);
                 // exits stay warp-uniform: the epilogue's tcgen05.ld is a warp-wide instruction
                 const bool w = bar_wait(&empty[s], ((it / kStages) & 1) ^ 1, s_abort, err);
                 if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
