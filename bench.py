@@ -139,8 +139,8 @@ def whole_job_rate(cells_per_rank: int, world: int, steps: int, ms_max: float) -
 # The sources that define the field-step kernels of the DM and SP pipelines
 # and their launch shapes (the per-kernel DRAM traffic in profiles/traffic.json
 # is valid while these are unchanged).
-STEP_KERNEL_SOURCES = ("fft_engine.cuh", "fft2.cuh", "xpipe.cuh", "zws.cuh", "sp.cuh", "passes_impl.cuh", "passes_f32.cu",
-                       "passes_f64.cu", "plan.h")
+STEP_KERNEL_SOURCES = ("fft_engine.cuh", "fft2.cuh", "mixed.cuh", "mix2.cuh", "xpipe.cuh", "zws.cuh", "zt.cuh", "sp.cuh",
+                       "spws.cuh", "passes_impl.cuh", "passes_f32.cu", "passes_f64.cu", "plan.h")
 
 
 def source_hash() -> str:
@@ -1193,7 +1193,8 @@ def run_reference(args, rank, world):
     print(json.dumps(out), flush=True)
 
 
-PASS_KERNELS = {"x_fwd": "k_x_fwd_tma", "y_fwd": "k_col3", "z_conv": "k_z_ws", "y_inv": "k_col3", "x_inv": "k_x_inv2"}
+PASS_KERNELS = {"x_fwd": "k_x_fwd2", "y_fwd": "k_mix2_col", "z_conv": "k_z_ws", "y_inv": "k_mix2_col",
+                "x_inv": "k_x_inv_bulk"}
 
 
 def write_traffic(logs, command, workload):
@@ -1201,7 +1202,7 @@ def write_traffic(logs, command, workload):
     dram__bytes_write.sum,gpu__time_duration.sum, one or two launches per log
     of the 256^3 step): per pass its kernel's DRAM bytes per launch and per
     cell, keyed by the hash of the step-kernel sources. The y passes share a
-    kernel template: the first captured k_col3 launch of a log is the forward
+    kernel template: the first captured k_mix2_col launch of a log is the forward
     pass, the second the inverse one."""
     import csv as _csv
     launches = []  # (kernel name, {metric: value}) in capture order
@@ -1216,10 +1217,10 @@ def write_traffic(logs, command, workload):
             ent[1][r[mi]] = float(r[vi].replace(",", ""))
         launches += [by_id[k] for k in sorted(by_id, key=int)]
     cells = N_GRID[0] * N_GRID[1] * N_GRID[2]
-    out, col3 = {}, [l for l in launches if "k_col3" in l[0]]
+    out, cols = {}, [l for l in launches if "k_mix2_col" in l[0]]
     for name, pat in PASS_KERNELS.items():
-        if pat == "k_col3":
-            pick = col3[0] if name == "y_fwd" and col3 else (col3[1] if len(col3) > 1 else None)
+        if pat == "k_mix2_col":
+            pick = cols[0] if name == "y_fwd" and cols else (cols[1] if len(cols) > 1 else None)
         else:
             pick = next((l for l in launches if pat in l[0]), None)
         if pick is None:
