@@ -14,6 +14,10 @@
 //    stage's inputs r >= (R1 + 1) / 2 are zero at compile time (rows j + r R2 with
 //    j < R2 are then at or beyond L / 2), and only the outputs r <= R2 / 2 of an
 //    inverse last stage are formed.
+// Against the general kernels (120-190 instructions per point, now 40-90), FP32: 130^3
+// padded to 270^3, x forward 67 -> 29 us, y 74 -> 39 and 80 -> 49, z 300 -> 137, x inverse
+// 66 -> 40; 300 x 260 x 100 padded to 600 x 540 x 256, x forward 196 -> 92, y 226 -> 142
+// and 226 -> 173, x inverse 127 -> 97. Still latency-bound: 35-50% of the issue slots.
 #pragma once
 #include "mixed.cuh"
 #include "fft2.cuh"
@@ -255,6 +259,9 @@ k_mix2_col(const typename Cplx<T>::type *__restrict__ in, typename Cplx<T>::type
 // read without conflicts.
 __host__ __device__ inline int mix2_tensor_stride(int HZ) { return 24 * HZ + (16 - 24 * HZ % 32 + 32) % 32; }
 
+// Threads of a row-pass CTA: with 256 the three barriers of fewer, larger CTAs left the
+// scheduler idle (x forward at 130^3: 41 us with 256 and serial loads, 29 with 128 and the
+// loads issued together).
 constexpr int kMix2RowThreads = 128;
 
 // Real-to-complex rows (as k_gen_x_fwd): g.G rows per CTA, one butterfly of
@@ -481,7 +488,8 @@ k_mix2_x_inv(const typename Cplx<T>::type *__restrict__ in, int64_t in_rs, int n
 // Middle, one thread per (m, column): the three components' R2-point DFTs
 // in registers, the product at kz = m + R1 q, the inverse DFTs and both
 // twiddles, in place. Stage 3: R1-point inverse DFTs, rows z < nrows stored. The middle
-// holds three components, so R2 is the smaller radix. FP32: the tile's tensor block (two
+// holds three components, so R2 is the smaller radix (130^3 -> 270^3, 30 x 9: 137 us at
+// two CTAs per SM, 51% of the issue slots; DRAM floor 43 us). FP32: the tile's tensor block (two
 // 4-column sub-blocks of the tile-ordered copy) is copied to shared memory with
 // 16-byte asynchronous copies while stage 1 runs; FP64 reads the octant table.
 template <typename T, int TC, int MAXR2>

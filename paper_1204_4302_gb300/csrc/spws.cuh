@@ -10,7 +10,7 @@
 // the 16 values of the current component, and the shared memory of a tile (input 48 KB,
 // exchange 33 KB, kernel block 25 KB at L = 512) admits two CTAs of 256 threads per
 // SM, whose phases overlap; k_sp_z2 held three exchange tiles and three components in
-// registers with one CTA of 384 threads per SM.
+// registers with one CTA of 384 threads per SM. 256^3: 782 -> 406 us (DRAM floor 190).
 #pragma once
 #include "zt.cuh"
 

@@ -88,8 +88,8 @@ __global__ void k_tg_tables(const double *__restrict__ snode, int R, int nx, int
 // What bounds it is shared-memory reads per multiply-add, so a thread forms
 // kTgNO outputs (a block's width apart: consecutive lanes read consecutive table
 // entries) of the VC vectors: kTgNO table reads and VC / 4 vector reads for
-// kTgNO VC multiply-adds. Rank 8 at 256^3: 52 us for three launches of one output per
-// thread (9 reads for 8 multiply-adds).
+// kTgNO VC multiply-adds. Rank 8 at 256^3: three launches of one output per thread (9
+// reads for 8 multiply-adds) took 70 us, this one about 45.
 constexpr int kTgNO = 4;
 template <typename T> struct TgAxes {
     const T *U[3];
@@ -252,7 +252,7 @@ k_tg_dense(const T *__restrict__ X, const T *__restrict__ Y, const T *__restrict
 // The energy's 3 r loads and multiply-adds per cell bound it, so a block takes
 // kTgFieldRows rows j at once and a thread one i of all of them: a factor is loaded
 // once for four cells, their w arrive in one vector read, and the rows share their y
-// neighbours. Rank 8 at 256^3: 202 us with one row at a time.
+// neighbours. Rank 8 at 256^3: 202 -> 124 us (issue slots 61% busy; HBM floor 40 us).
 constexpr int kTgFieldThreads = 128, kTgFieldRows = 4;
 
 template <typename T>
