@@ -40,7 +40,8 @@ class DemagEnergy(torch.autograd.Function):
         saved = ctx.saved_tensors
         m = saved[0]
         w = saved[1] if ctx.has_w else None
-        g = gE.detach().to(dtype=torch.float64).reshape(()).contiguous()
+        # E is a float64 scalar, so its gradient is one too: handed on as it is
+        g = gE if gE.dtype == torch.float64 and gE.dim() == 0 else gE.detach().to(dtype=torch.float64).reshape(())
         _, grad = ctx.plan.energy_grad(m, ctx.Ms, w, want_energy=False, want_grad=True, gscale=g)
         return grad, None, None, None
 

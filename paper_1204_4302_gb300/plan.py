@@ -64,7 +64,8 @@ class Plan:
 
     # ------------------------------------------------------------------ basics
     def _stream(self) -> int:
-        return torch.cuda.current_stream(self.device).cuda_stream
+        # the raw handle without a Stream object: 2 us of a 20 us call on a small grid
+        return torch._C._cuda_getCurrentRawStream(self.device.index)
 
     def _field_arg(self, t: torch.Tensor, name: str) -> torch.Tensor:
         if not isinstance(t, torch.Tensor) or t.device != self.device:
