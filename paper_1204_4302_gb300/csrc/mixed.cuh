@@ -4,9 +4,10 @@
 // next power of two (e.g. n = 80: 160 instead of 256 per axis). These kernels
 // trade the compile-time register schedules of the power-of-two passes for
 // one generic form: a tile of transforms in shared memory, Stockham stages
-// of any radix R <= 32 with prime factors 2, 3, 5, 7 (in-register DFTs with
+// of any radix R <= 16 (FP32 z passes: <= 32 where that saves a stage, see
+// gen_z_radix) with prime factors 2, 3, 5, 7 (in-register DFTs with
 // compile-time twiddles) run from a runtime radix list, ping-ponging between
-// two buffers; most lengths take two stages, like the power-of-two passes.
+// two buffers.
 // Same inputs, outputs and epilogues as the power-of-two passes.
 #pragma once
 #include <type_traits>
@@ -221,7 +222,10 @@ template <int R, bool INV, typename C> struct MixDFT {
     }
 };
 
-constexpr int kGenMaxRadixRows = 16, kGenMaxRadixZ = 16;
+constexpr int kGenMaxRadixRows = 16;
+// smallest radix that the kernels of largest radix 32 hold (their plans, lengths
+// above 128 in as few stages as radices <= 32 allow, need no smaller one)
+__host__ __device__ constexpr int gen_min_radix(int maxr) { return maxr > 16 ? 9 : 2; }
 
 // Stages with caller-supplied ends: the first stage reads its inputs through
 // ld(row, col) (global memory, with the pass's prologue) and the last stage
@@ -288,14 +292,15 @@ template <typename C, bool INV, bool XROW, int MAXR, typename LD, typename ST>
 __device__ __forceinline__ void gen_stage_any(const GenRadix &g, int s, const C *__restrict__ tw, int twstride,
                                               const LD &ld, const ST &st)
 {
+    constexpr int MINR = gen_min_radix(MAXR);
     switch (g.r[s]) {
-    case 2: gen_stage_io<C, 2, INV, XROW>(g, s, tw, twstride, ld, st); break;
-    case 3: gen_stage_io<C, 3, INV, XROW>(g, s, tw, twstride, ld, st); break;
-    case 4: gen_stage_io<C, 4, INV, XROW>(g, s, tw, twstride, ld, st); break;
-    case 5: gen_stage_io<C, 5, INV, XROW>(g, s, tw, twstride, ld, st); break;
-    case 6: gen_stage_io<C, 6, INV, XROW>(g, s, tw, twstride, ld, st); break;
-    case 7: gen_stage_io<C, 7, INV, XROW>(g, s, tw, twstride, ld, st); break;
-    case 8: gen_stage_io<C, 8, INV, XROW>(g, s, tw, twstride, ld, st); break;
+    case 2: if constexpr (MINR <= 2) gen_stage_io<C, 2, INV, XROW>(g, s, tw, twstride, ld, st); break;
+    case 3: if constexpr (MINR <= 3) gen_stage_io<C, 3, INV, XROW>(g, s, tw, twstride, ld, st); break;
+    case 4: if constexpr (MINR <= 4) gen_stage_io<C, 4, INV, XROW>(g, s, tw, twstride, ld, st); break;
+    case 5: if constexpr (MINR <= 5) gen_stage_io<C, 5, INV, XROW>(g, s, tw, twstride, ld, st); break;
+    case 6: if constexpr (MINR <= 6) gen_stage_io<C, 6, INV, XROW>(g, s, tw, twstride, ld, st); break;
+    case 7: if constexpr (MINR <= 7) gen_stage_io<C, 7, INV, XROW>(g, s, tw, twstride, ld, st); break;
+    case 8: if constexpr (MINR <= 8) gen_stage_io<C, 8, INV, XROW>(g, s, tw, twstride, ld, st); break;
     case 9: gen_stage_io<C, 9, INV, XROW>(g, s, tw, twstride, ld, st); break;
     case 10: gen_stage_io<C, 10, INV, XROW>(g, s, tw, twstride, ld, st); break;
     case 12: gen_stage_io<C, 12, INV, XROW>(g, s, tw, twstride, ld, st); break;
@@ -508,7 +513,8 @@ k_gen_x_inv(const typename Cplx<T>::type *__restrict__ in, int64_t in_rs, int nr
 // with the first stage reading global memory (rows < nrows), the 3x3
 // product with the folded tensor spectrum in shared memory, inverse
 // transform whose last stage stores rows < nrows. Column f = ky * width + kx.
-template <typename T>
+// MAXR: the largest stage radix (gen_z_radix).
+template <typename T, int MAXR>
 __global__ void __launch_bounds__(kGenThreads)
 k_gen_zconv(typename Cplx<T>::type *__restrict__ S, int ncols, int width, unsigned mw, int64_t ss, int64_t rs,
             int64_t cs, int nrows, const T *__restrict__ nhat, int Py, int Kx,
@@ -532,7 +538,7 @@ k_gen_zconv(typename Cplx<T>::type *__restrict__ S, int ncols, int width, unsign
         return ok ? S[q] : cmk<C>(0, 0);
     };
     const GenSmemSt<C, false> none{nullptr, TCC, L};
-    C *F = gen_fft_io<C, false, false, false, kGenMaxRadixZ>(A, B, g, tw, twstride, ld, none);
+    C *F = gen_fft_io<C, false, false, false, MAXR>(A, B, g, tw, twstride, ld, none);
     C *G = F == A ? B : A;
     const int hy = Py / 2 + 1, hz = L / 2 + 1;
     const int64_t plane = (int64_t)hz * hy * Kx;
@@ -561,7 +567,7 @@ k_gen_zconv(typename Cplx<T>::type *__restrict__ S, int ncols, int width, unsign
         const int64_t q = gaddr(row, cc, ok);
         if (ok) S[q] = v;
     };
-    gen_fft_io<C, true, false, true, kGenMaxRadixZ>(G, F, g, tw, twstride, GenSmemLd<C, false>{F, TCC, L}, st);
+    gen_fft_io<C, true, false, true, MAXR>(G, F, g, tw, twstride, GenSmemLd<C, false>{F, TCC, L}, st);
 }
 
 // Fused SP z pass (as k_sp_z2) for lengths that are not powers of two: the
@@ -571,8 +577,8 @@ k_gen_zconv(typename Cplx<T>::type *__restrict__ S, int ncols, int width, unsign
 // columns; its inverse transform (plan g1, TC columns) stores the nout = nrows
 // + 1 node rows over component 0 (running on into the first row of component
 // 1, cs == nrows * rs: only this CTA reads or writes its columns, and every
-// input was read before the first output is written).
-template <typename T>
+// input was read before the first output is written). MAXR as in k_gen_zconv.
+template <typename T, int MAXR>
 __global__ void __launch_bounds__(kGenThreads)
 k_gen_sp_zconv(typename Cplx<T>::type *__restrict__ S, int ncols, int width, unsigned mw, int64_t ss, int64_t rs,
                int64_t cs, int nrows, int nout, const T *__restrict__ that, int Py, int Kx,
@@ -595,7 +601,7 @@ k_gen_sp_zconv(typename Cplx<T>::type *__restrict__ S, int ncols, int width, uns
         return v;
     };
     const GenSmemSt<C, false> none{nullptr, TCC, L};
-    C *F = gen_fft_io<C, false, false, false, kGenMaxRadixZ>(A, B, g3, tw, 1, ld, none);
+    C *F = gen_fft_io<C, false, false, false, MAXR>(A, B, g3, tw, 1, ld, none);
     C *G = F == A ? B : A;
     const int hy = Py / 2 + 1, hz = L / 2 + 1;
     const int64_t plane = (int64_t)hz * hy * Kx;
@@ -628,7 +634,7 @@ k_gen_sp_zconv(typename Cplx<T>::type *__restrict__ S, int ncols, int width, uns
             S[(int64_t)slab * ss + (int64_t)row * rs + (f - slab * width)] = v;
         }
     };
-    gen_fft_io<C, true, false, true, kGenMaxRadixZ>(G, F, g1, tw, 1, ldf, st);
+    gen_fft_io<C, true, false, true, MAXR>(G, F, g1, tw, 1, ldf, st);
 }
 
 }  // namespace demag

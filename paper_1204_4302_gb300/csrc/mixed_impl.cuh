@@ -85,6 +85,20 @@ bool gen_plan(int L, int tile, GenRadix &g, int maxr, int comps = 1)
     return true;
 }
 
+// Largest stage radix of the general z passes. FP32: 32 where that saves a stage
+// against 16 above length 128 (an exchange and a barrier per direction; us of the z pass
+// with 16 and with 32: SP 200^3 106 / 97, 270^3 267 / 224, 300^3 371 / 319, DM
+// 128 x 128 x 600 207 / 185), else 16, whose kernel is the smaller (SP 120^3 26.7, 28.6
+// with 32). FP64: 16, as a thread of the larger radices holds twice the registers
+// (SP 200^3 1068, 1523 with 32; 300^3 4194, 5938).
+template <typename T> int gen_z_radix(int L)
+{
+    if (sizeof(T) == 8 || L <= 128) return 16;
+    GenRadix a, b;
+    const bool big = gen_plan(L, gen_tile_elems<T>(true), b, 32, 3) && b.r[b.n - 1] >= gen_min_radix(32);
+    return big && !(gen_plan(L, gen_tile_elems<T>(true), a, 16, 3) && a.n <= b.n) ? 32 : 16;
+}
+
 // Two-stage plan L = R1 R2 with radices <= maxr: the smallest largest radix,
 // the larger one first (forward: its inputs are half empty) or last (inverse: half
 // of its outputs are not formed). False where L has no such split.
@@ -195,6 +209,46 @@ cudaError_t mix2_z_launch(typename Cplx<T>::type *S, int Kx, int Py, int64_t ss,
 }
 
 }  // namespace
+
+template <typename T, int MAXR>
+cudaError_t gen_z_launch(int L, typename Cplx<T>::type *S, int ncols, int width, int64_t ss, int64_t rs, int64_t cs, int nrows,
+                         const T *nhat, int Py, int Kx, const typename Cplx<T>::type *tw, int twstride, cudaStream_t st)
+{
+    GenRadix g;
+    if (!gen_plan(L, gen_tile_elems<T>(true), g, MAXR, 3)) return cudaErrorInvalidValue;
+    const int cols = g.TC / 3;
+    const size_t sm = 2 * swsize(L * g.TC) * sizeof(typename Cplx<T>::type);
+    cudaError_t e = allow_smem<k_gen_zconv<T, MAXR>>(sm);
+    if (e != cudaSuccess) return e;
+    k_gen_zconv<T, MAXR><<<(ncols + cols - 1) / cols, kGenThreads, sm, st>>>(
+        S, ncols, width, magic_of(width), ss, rs, cs, nrows, nhat, Py, Kx, tw, twstride, g);
+    return cudaGetLastError();
+}
+
+template <typename T, int MAXR>
+cudaError_t gen_sp_z_launch(int L, typename Cplx<T>::type *S, int ncols, int width, int64_t ss, int64_t rs, int64_t cs,
+                            int nrows, int nout, const T *that, int Py, int Kx, const typename Cplx<T>::type *tw,
+                            const typename Cplx<T>::type *phx, const typename Cplx<T>::type *phy,
+                            const typename Cplx<T>::type *phz, cudaStream_t st)
+{
+    GenRadix g3, g1;
+    if (!gen_plan(L, gen_tile_elems<T>(true), g3, MAXR, 3)) return cudaErrorInvalidValue;
+    if (!gen_plan(L, gen_tile_elems<T>(true), g1, MAXR, 1)) return cudaErrorInvalidValue;
+    const int cols = g1.TC;
+    const size_t sm = 2 * swsize(L * g3.TC) * sizeof(typename Cplx<T>::type);
+    cudaError_t e = allow_smem<k_gen_sp_zconv<T, MAXR>>(sm);
+    if (e != cudaSuccess) return e;
+    k_gen_sp_zconv<T, MAXR><<<(ncols + cols - 1) / cols, kGenThreads, sm, st>>>(
+        S, ncols, width, magic_of(width), ss, rs, cs, nrows, nout, that, Py, Kx, tw, phx, phy, phz, g3, g1);
+    return cudaGetLastError();
+}
+
+// the FP32 kernels of largest radix 32: a translation unit of their own (compile time)
+extern template cudaError_t gen_z_launch<float, 32>(int, float2 *, int, int, int64_t, int64_t, int64_t, int, const float *,
+                                                    int, int, const float2 *, int, cudaStream_t);
+extern template cudaError_t gen_sp_z_launch<float, 32>(int, float2 *, int, int, int64_t, int64_t, int64_t, int, int,
+                                                       const float *, int, int, const float2 *, const float2 *,
+                                                       const float2 *, const float2 *, cudaStream_t);
 
 template <typename T>
 bool MixedPasses<T>::z_tiled(int L)
@@ -321,15 +375,10 @@ cudaError_t MixedPasses<T>::zconv(int L, C *S, int ncols, int width, int64_t ss,
         (sizeof(T) != 4 || (ntile && ((uintptr_t)ntile & 15) == 0)) && mix2_zsplit(L, m))
         return m.R2 <= 10 ? mix2_z_launch<T, 10>(S, Kx, Py, ss, rs, cs, nrows, nhat, ntile, tw, m, st)
                           : mix2_z_launch<T, 16>(S, Kx, Py, ss, rs, cs, nrows, nhat, ntile, tw, m, st);
-    GenRadix g;
-    if (!gen_plan(L, gen_tile_elems<T>(true), g, kGenMaxRadixZ, 3)) return cudaErrorInvalidValue;
-    const int cols = g.TC / 3;
-    const size_t sm = 2 * swsize(L * g.TC) * sizeof(C);
-    cudaError_t e = allow_smem<k_gen_zconv<T>>(sm);
-    if (e != cudaSuccess) return e;
-    k_gen_zconv<T><<<(ncols + cols - 1) / cols, kGenThreads, sm, st>>>(S, ncols, width, magic_of(width), ss, rs, cs,
-                                                                       nrows, nhat, Py, Kx, tw, twstride, g);
-    return cudaGetLastError();
+    if constexpr (sizeof(T) == 4)
+        if (gen_z_radix<T>(L) == 32)
+            return gen_z_launch<T, 32>(L, S, ncols, width, ss, rs, cs, nrows, nhat, Py, Kx, tw, twstride, st);
+    return gen_z_launch<T, 16>(L, S, ncols, width, ss, rs, cs, nrows, nhat, Py, Kx, tw, twstride, st);
 }
 
 template <typename T>
@@ -339,17 +388,10 @@ cudaError_t MixedPasses<T>::sp_zconv(int L, C *S, int ncols, int width, int64_t 
 {
     if (ncols <= 0) return cudaSuccess;
     if (2 * nrows > L || nout != nrows + 1 || cs != (int64_t)nrows * rs) return cudaErrorInvalidValue;
-    GenRadix g3, g1;
-    if (!gen_plan(L, gen_tile_elems<T>(true), g3, kGenMaxRadixZ, 3)) return cudaErrorInvalidValue;
-    if (!gen_plan(L, gen_tile_elems<T>(true), g1, kGenMaxRadixZ, 1)) return cudaErrorInvalidValue;
-    const int cols = g1.TC;
-    const size_t sm = 2 * swsize(L * g3.TC) * sizeof(C);
-    cudaError_t e = allow_smem<k_gen_sp_zconv<T>>(sm);
-    if (e != cudaSuccess) return e;
-    k_gen_sp_zconv<T><<<(ncols + cols - 1) / cols, kGenThreads, sm, st>>>(S, ncols, width, magic_of(width), ss, rs,
-                                                                          cs, nrows, nout, that, Py, Kx, tw, phx, phy,
-                                                                          phz, g3, g1);
-    return cudaGetLastError();
+    if constexpr (sizeof(T) == 4)
+        if (gen_z_radix<T>(L) == 32)
+            return gen_sp_z_launch<T, 32>(L, S, ncols, width, ss, rs, cs, nrows, nout, that, Py, Kx, tw, phx, phy, phz, st);
+    return gen_sp_z_launch<T, 16>(L, S, ncols, width, ss, rs, cs, nrows, nout, that, Py, Kx, tw, phx, phy, phz, st);
 }
 
 }  // namespace demag
