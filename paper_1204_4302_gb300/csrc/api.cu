@@ -1571,8 +1571,11 @@ demag_status demag_autotune(demag_plan_t p, int use_cache, double *best_ms, void
     if (z2 && dm && p->Pz >= 64 && p->Pz <= 512) zs.push_back(3);  // persistent, pipelined
     if (z2 && dm && p->Pz >= 32 && p->Pz <= 512) zs.push_back(4);   // half tile, two CTAs per SM
     if (z2 && dm && p->Pz >= 32 && p->Pz <= 128) zs.push_back(8);   // 8-point second stage, two CTAs per SM
-    if (z2 && p->Pz >= 32 && p->Pz <= 256) zs.push_back(5);   // persistent, TMA-staged input (DM and SP)
-    if (dm && p->ntile) {  // persistent, TMA input and tensor tiles, FP32: 8 or 4 columns per tile
+    // persistent, TMA-staged input (DM and SP; FP32 SP plans of length 256 have one form)
+    if (z2 && p->Pz >= 32 && p->Pz <= 256 && (dm || p->prec == DEMAG_F64 || p->Pz < 256)) zs.push_back(5);
+    // persistent, TMA input and tensor tiles, FP32: 8 or 4 columns per tile (other lengths
+    // hold a tile-ordered tensor copy too, for forms of their own)
+    if (dm && p->ntile && (p->Pz == 256 || p->Pz == 512)) {
         zs.push_back(6);
         zs.push_back(7);
     }
