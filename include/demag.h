@@ -402,10 +402,12 @@ demag_status demag_batch_status(demag_batch_t batch, void *stream);
 demag_status demag_batch_info(demag_batch_t batch, int *mode, int *persistent_ok, int *items, int *grid,
                               size_t *smem);
 
-/* Autotunes every state's plan (demag_autotune), then times the persistent
- * and the branch mode on temporary fields and keeps the faster mode.
- * ms_persistent / ms_branches (may be NULL) receive the time per call of each
- * mode (-1 when the persistent mode is unavailable). Synchronises. */
+/* Autotunes every state's plan (demag_autotune), then times the three modes on
+ * temporary fields and keeps the fastest; the pass-batched mode instead of the
+ * branches where these are less than a tenth faster (their graph is rebuilt
+ * whenever a call brings other buffers). ms_persistent / ms_branches (may be
+ * NULL) receive the time per call of these modes (-1 when the persistent mode
+ * is unavailable). Synchronises. */
 demag_status demag_batch_autotune(demag_batch_t batch, int use_cache, double *ms_persistent,
                                   double *ms_branches, void *stream);
 
@@ -415,7 +417,8 @@ demag_status demag_batch_autotune(demag_batch_t batch, int use_cache, double *ms
  * faster of the two (rebuilding the batch's plans in place when the other
  * wins; the handle stays valid, graphs are rebuilt at the next call, and a
  * timeout set with demag_batch_set_timeout returns to its default).
- * ms_pow2 / ms_smooth (may be NULL) receive the best time per call of each.
+ * ms_pow2 / ms_smooth (may be NULL) receive the time per call of each, in the
+ * mode that demag_batch_autotune keeps for it; the two are compared by it.
  * DEMAG_ERR_UNSUPPORTED for a batch created with DEMAG_PAD_TUNED.
  * Synchronises. */
 demag_status demag_batch_autotune_padding(demag_batch_t batch, int use_cache, double *ms_pow2, double *ms_smooth,

@@ -49,13 +49,14 @@ class Batch:
 
     def autotune(self, use_cache: bool = True):
         """Tune every state's plan and choose the fastest batch mode (persistent,
-        branches, pass-batched); returns (ms per call persistent, ms per call
-        branches)."""
+        branches, pass-batched; branches only where a tenth faster than
+        pass-batched, as their graph is rebuilt for other buffers); returns (ms
+        per call persistent, ms per call branches)."""
         return B.demag_batch_autotune(self.handle, use_cache, torch.cuda.current_stream(self.device).cuda_stream)
 
     def autotune_padding(self, use_cache: bool = True):
-        """Keep the faster of power-of-two and smooth padding (rebuilding the
-        plans when needed); returns (ms per call power-of-two, smooth)."""
+        """Keep the faster of power-of-two and smooth padding, each in the mode
+        that autotune chooses for it (rebuilding the plans when needed); returns (ms per call power-of-two, smooth)."""
         return B.demag_batch_autotune_padding(self.handle, use_cache, torch.cuda.current_stream(self.device).cuda_stream)
 
     def set_mode(self, mode: int):

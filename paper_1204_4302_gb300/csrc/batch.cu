@@ -30,6 +30,7 @@
 #include <utility>
 #include <vector>
 
+#include "batch_mode.h"
 #include "fft2.cuh"
 #include "zt.cuh"
 #include "plan.h"
@@ -1113,13 +1114,7 @@ demag_status demag_batch_autotune(demag_batch_t b, int use_cache, double *ms_per
     b->timing = timing;
     release();
     if (rs != DEMAG_OK) return rs;
-    // the branch graph is rebuilt whenever a call brings other buffers (6 ms for 64
-    // states against a call of 1.4 ms), the other modes upload a table: it is taken
-    // where it is faster by a tenth
-    int best = b->persistent_ok ? 2 : 1;
-    if (t[0] < t[best]) best = 0;
-    if (t[1] < 0.9 * t[best]) best = 1;
-    b->mode = best;
+    b->mode = demag::batch_pick_mode(t);
     b->tuned_ms[0] = t[0]; b->tuned_ms[1] = t[1]; b->tuned_ms[2] = t[2];
     if (ms_persistent) *ms_persistent = b->persistent_ok ? t[0] : -1.0;
     if (ms_branches) *ms_branches = t[1];
@@ -1135,7 +1130,7 @@ demag_status demag_batch_autotune_padding(demag_batch_t b, int use_cache, double
     double tp = 0, tb = 0;
     demag_status s = demag_batch_autotune(b, use_cache, &tp, &tb, stream);
     if (s != DEMAG_OK) return s;
-    const double t_this = std::min(b->tuned_ms[0], std::min(b->tuned_ms[1], b->tuned_ms[2]));
+    const double t_this = b->tuned_ms[b->mode];  // of the mode that is kept
     demag_options o;
     memset(&o, 0, sizeof o);
     o.pad_mode = b->pad_mode == DEMAG_PAD_POW2 ? DEMAG_PAD_SMOOTH : DEMAG_PAD_POW2;
@@ -1147,7 +1142,7 @@ demag_status demag_batch_autotune_padding(demag_batch_t b, int use_cache, double
         free_batch(nb);
         return s;
     }
-    const double t_other = std::min(nb->tuned_ms[0], std::min(nb->tuned_ms[1], nb->tuned_ms[2]));
+    const double t_other = nb->tuned_ms[nb->mode];
     const bool was_pow2 = b->pad_mode == DEMAG_PAD_POW2;
     if (ms_pow2) *ms_pow2 = was_pow2 ? t_this : t_other;
     if (ms_smooth) *ms_smooth = was_pow2 ? t_other : t_this;
