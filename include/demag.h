@@ -100,7 +100,8 @@ demag_status demag_plan_load(const char *path, demag_plan_t *out);
 /* Test hook for the error paths: with n >= 1 the n-th next device allocation
  * made by plan creation, tensor setup, the host-buffer entry points or the
  * autotuner fails as if the device were out of memory (the call returns
- * DEMAG_ERR_OOM and frees what it had allocated); 0 disarms it. */
+ * DEMAG_ERR_OOM and frees what it had allocated; a plan goes without its
+ * tile-ordered copy, see demag_tensor_setup); 0 disarms it. */
 void demag_debug_fail_alloc(long n);
 
 /* Debug allocations: with DEMAG_DEBUG=1 in the environment, every device
@@ -206,7 +207,12 @@ demag_status demag_sp_potential(demag_plan_t plan, const void *M, void *phi, voi
  * kernel at intermediate range, a multipole expansion of the cell average
  * far away), places them at wrapped offsets of the padded grid and stores
  * the (real) 3-D spectrum. Allocates and frees temporary device memory;
- * blocks until done. Idempotent. */
+ * blocks until done. Idempotent.
+ * FP32 plans whose z length is 32 to 512, or a mixed-radix one in two stages (SP:
+ * 256 and 512), also keep a copy of the spectrum in the order their z pass
+ * reads it, about as large again (counted in demag_info.device_bytes). Where
+ * the device has no memory left for it the plan works without, by slower z
+ * forms; batches of such plans run as branches only. */
 demag_status demag_tensor_setup(demag_plan_t plan, void *stream);
 
 /* H = -N * M (paper Sec. 3.1, Eq. "demag"). M, H: device, [3][nz][ny][nx] of

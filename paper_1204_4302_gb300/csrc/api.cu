@@ -360,8 +360,9 @@ demag_status run_field(demag_plan *p, const FieldJob &job, cudaStream_t st)
     cudaError_t e;
     // energy without a field: the spectral (Parseval) sum in the z pass,
     // E = (mu0/2) (V / (Px Py Pz)) sum_k w(kx) M^H N^ M, no inverse passes
+    // (FP32 at z lengths 32 to 128 reads the tile-ordered tensor copy for it)
     const bool spectral = !job.out && job.E_dev && p->spectral_energy &&
-                          Passes<T>::zenergy_blocks(Pz, Py, Kx) > 0;
+                          Passes<T>::zenergy_blocks(Pz, Py, Kx) > 0 && (!f32 || p->ntile || Pz < 32 || Pz > 128);
     // x forward
     if (Px == 1) e = Passes<T>::x1_fwd(xi, rows, S1, st);
     else e = Passes<T>::x_fwd(Px / 2, xi, rows, nx, S1, Kxp, twx, st, p->xvariant);
@@ -906,9 +907,11 @@ size_t table_count(const demag_plan *p)
     return (size_t)(p->method == DEMAG_METHOD_SP ? 3 : 6) * plane;
 }
 
-// The tile-ordered copy of the FP32 tensor spectrum read by the persistent
-// TMA z pass (z variant 6), built from nhat32 on the plan's stream; plans whose
-// z length that kernel does not support keep none.
+// The tile-ordered copy of an FP32 plan's tables, built from nhat32 on the
+// plan's stream: read by the persistent TMA z passes (z length 256 and 512, SP too),
+// the small-tile z pass (32 to 128) and the two-stage mixed-radix z pass; other
+// lengths keep none. Every one of these has a form that reads nhat32 itself, so where
+// the device has no memory left for the copy the plan goes without.
 cudaError_t build_ntile(demag_plan *p, cudaStream_t st)
 {
     if (p->prec != DEMAG_F32 || !p->nhat32) return cudaSuccess;
@@ -919,12 +922,21 @@ cudaError_t build_ntile(demag_plan *p, cudaStream_t st)
         cudaError_t e = dmalloc(&p->ntile, n * sizeof(float));
         if (e != cudaSuccess) {
             p->ntile = nullptr;
-            return e;
+            if (e != cudaErrorMemoryAllocation) return e;
+            cudaGetLastError();
+            return cudaSuccess;
         }
         p->ntile_bytes = n * sizeof(float);
         p->device_bytes += p->ntile_bytes;
     }
     return Passes<float>::tile_tensor(p->Pz, p->nhat32, p->ntile, p->Py, p->Kx, st, sp);
+}
+
+// Whether the plan goes without a tile-ordered copy that its lengths have a use for.
+bool ntile_missing(const demag_plan *p)
+{
+    return p->prec == DEMAG_F32 && !p->ntile &&
+           Passes<float>::tile_tensor_elems(p->Pz, p->Py, p->Kx, p->method == DEMAG_METHOD_SP) > 0;
 }
 
 // A plan that is only timed (padding autotuner): its tensor spectrum is
@@ -1141,15 +1153,21 @@ demag_status sp_setup(demag_plan *p, cudaStream_t st)
                                        (int64_t)Py * Kxp, Pz, p->tw64[2], 1, st));
         SETUP_CUDA(demag::sp_extract(St, c, Px, Py, Pz, Kxp, t64, p->nhat32, imag, st));
     }
-    SETUP_CUDA(build_ntile(p, st));
     unsigned long long bits = 0;
     SETUP_CUDA(cudaMemcpyAsync(&bits, imag, sizeof(bits), cudaMemcpyDeviceToHost, st));
     SETUP_CUDA(cudaStreamSynchronize(st));
     memcpy(&p->imag_max, &bits, sizeof(double));
+    done(DEMAG_OK);  // the temporaries make room for the tile-ordered copy
+    oct = W = nullptr;
+    St = nullptr;
+    imag = nullptr;
+    own64 = false;
+    SETUP_CUDA(build_ntile(p, st));
+    SETUP_CUDA(cudaStreamSynchronize(st));
     p->launches += 1 + 3 * 5;
     p->setup_done = true;
     g_err.clear();
-    return done(DEMAG_OK);
+    return DEMAG_OK;
 #undef SETUP_CUDA
 }
 
@@ -1211,15 +1229,21 @@ demag_status demag_tensor_setup(demag_plan_t p, void *stream)
                                            (int64_t)Py * Kxp, Pz, p->tw64[2], 1, st));
         SETUP_CUDA(demag::tensor_extract(St, c, Px, Py, Pz, Kxp, nh64, p->nhat32, imag, st));
     }
-    SETUP_CUDA(build_ntile(p, st));
     unsigned long long bits = 0;
     SETUP_CUDA(cudaMemcpyAsync(&bits, imag, sizeof(bits), cudaMemcpyDeviceToHost, st));
     SETUP_CUDA(cudaStreamSynchronize(st));
     memcpy(&p->imag_max, &bits, sizeof(double));
+    done(DEMAG_OK);  // the temporaries make room for the tile-ordered copy
+    oct = W = nullptr;
+    St = nullptr;
+    imag = nullptr;
+    own64 = false;
+    SETUP_CUDA(build_ntile(p, st));
+    SETUP_CUDA(cudaStreamSynchronize(st));
     p->launches += 1 + 6 * (2 + (Py > 1) + (Pz > 1));
     p->setup_done = true;
     g_err.clear();
-    return done(DEMAG_OK);
+    return DEMAG_OK;
 #undef SETUP_CUDA
 }
 
@@ -1570,9 +1594,10 @@ demag_status demag_autotune(demag_plan_t p, int use_cache, double *best_ms, void
     if (z2 && dm && p->Pz == 512) zs.push_back(2);  // 256 threads: the product stage uses every thread
     if (z2 && dm && p->Pz >= 64 && p->Pz <= 512) zs.push_back(3);  // persistent, pipelined
     if (z2 && dm && p->Pz >= 32 && p->Pz <= 512) zs.push_back(4);   // half tile, two CTAs per SM
-    if (z2 && dm && p->Pz >= 32 && p->Pz <= 128) zs.push_back(8);   // 8-point second stage, two CTAs per SM
+    if (z2 && dm && p->Pz >= 32 && p->Pz <= 128 && (p->ntile || p->prec == DEMAG_F64))
+        zs.push_back(8);  // 8-point second stage: small tiles (FP32), two CTAs per SM (FP64)
     // persistent, TMA-staged input (DM and SP; FP32 SP plans of length 256 have one form)
-    if (z2 && p->Pz >= 32 && p->Pz <= 256 && (dm || p->prec == DEMAG_F64 || p->Pz < 256)) zs.push_back(5);
+    if (z2 && p->Pz >= 32 && p->Pz <= 256 && (dm || !p->ntile || p->Pz < 256)) zs.push_back(5);
     // persistent, TMA input and tensor tiles, FP32: 8 or 4 columns per tile (other lengths
     // hold a tile-ordered tensor copy too, for forms of their own)
     if (dm && p->ntile && (p->Pz == 256 || p->Pz == 512)) {
@@ -1631,7 +1656,8 @@ demag_status demag_autotune(demag_plan_t p, int use_cache, double *best_ms, void
     p->xvariant = bx;
     p->tuned = true;
     if (best_ms) *best_ms = best;
-    if (use_cache) tune_store(key, bz, by, bx, best);
+    // (not for plans of these sizes that have their tile-ordered copy)
+    if (use_cache && !ntile_missing(p)) tune_store(key, bz, by, bx, best);
     return DEMAG_OK;
 }
 
@@ -1672,6 +1698,7 @@ demag_status demag_tune_padding(int nx, int ny, int nz, double dx, double dy, do
     }
     double tbest = 1e30, tpow2 = -1;
     int bP[3] = {0, 0, 0};
+    bool complete = true;  // every candidate was timed with its tile-ordered copy
     for (int i : cand[0])
         for (int j : cand[1])
             for (int k : cand[2]) {
@@ -1683,6 +1710,7 @@ demag_status demag_tune_padding(int nx, int ny, int nz, double dx, double dy, do
                 double ms = 0;
                 if (s == DEMAG_OK) s = zero_spectrum_for_timing(p, (cudaStream_t)stream);
                 if (s == DEMAG_OK) s = demag_autotune(p, use_cache, &ms, stream);
+                if (s == DEMAG_OK && ntile_missing(p)) complete = false;
                 demag_plan_destroy(p);
                 if (s != DEMAG_OK) return s;
                 if (i == cand[0][0] && j == cand[1][0] && k == cand[2][0]) tpow2 = ms;
@@ -1695,7 +1723,7 @@ demag_status demag_tune_padding(int nx, int ny, int nz, double dx, double dy, do
     best->px = bP[0]; best->py = bP[1]; best->pz = bP[2];
     if (ms_best) *ms_best = tbest;
     if (ms_pow2) *ms_pow2 = tpow2;
-    if (use_cache) {
+    if (use_cache && complete) {
         tune_store(kbest, bP[0], bP[1], bP[2], tbest);
         tune_store(kpow2, cand[0][0], cand[1][0], cand[2][0], tpow2);
     }

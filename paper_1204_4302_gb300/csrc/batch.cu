@@ -545,6 +545,10 @@ demag_status build_persistent(demag_batch *b)
             b->why_not_persistent = "state " + std::to_string(i) + " has transform lengths outside the persistent kernel";
             return DEMAG_OK;
         }
+        if (demag::zt_batch_items(b->plans[i]->Pz, b->plans[i]->Py, b->plans[i]->Kx) && !b->plans[i]->ntile) {
+            b->why_not_persistent = "state " + std::to_string(i) + " has no tile-ordered tensor copy (device memory)";
+            return DEMAG_OK;
+        }
         for (int k = 0; k < demag::kPasses; ++k)
             if (geo[i].tiles[k] > 0 && geo[i].smem[k] > smem) smem = geo[i].smem[k];
         npart += (size_t)std::max(geo[i].tiles[4], demag::zt_batch_items(b->plans[i]->Pz, b->plans[i]->Py, b->plans[i]->Kx));
