@@ -441,13 +441,12 @@ demag_status run_field(demag_plan *p, const FieldJob &job, cudaStream_t st)
     }
     tm.mark();
     // x inverse (+ epilogue)
-    int nblocks;
+    int nblocks = 0;
     if (Px == 1) {
         nblocks = p->npartials;
         e = Passes<T>::x1_inv(S1, rows, xo, nblocks, st);
     } else {
-        nblocks = Passes<T>::x_blocks(Px / 2, rows, p->xvariant);
-        e = Passes<T>::x_inv(Px / 2, S1, Kxp, rows, nx, xo, twx, st, p->xvariant);
+        e = Passes<T>::x_inv(Px / 2, S1, Kxp, rows, nx, xo, twx, st, p->xvariant, &nblocks);
     }
     if (e != cudaSuccess) return fail(DEMAG_ERR_CUDA, std::string("x inverse: ") + cudaGetErrorString(e));
     p->launches++;

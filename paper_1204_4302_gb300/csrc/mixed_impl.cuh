@@ -302,15 +302,17 @@ int MixedPasses<T>::x_blocks(int L, int nrows)
 
 template <typename T>
 cudaError_t MixedPasses<T>::x_inv(int L, const C *in, int64_t in_rs, int nrows, int nvalid, const XOut<T> &o,
-                                  const C *twx, cudaStream_t st)
+                                  const C *twx, cudaStream_t st, int *blocks)
 {
+    int unused, &grid = blocks ? *blocks : unused;
+    grid = 0;
     if (nrows <= 0) return cudaSuccess;
     Mix2 m;
     if (mix2_split(L, kMix2RowRadix, false, m)) {
         if (nvalid > L + 1) return cudaErrorInvalidValue;
         mix2_rows(m);
         const size_t sm = (size_t)m.G * m.R2 * m.RP * sizeof(C);
-        const int grid = (nrows + m.G - 1) / m.G;
+        grid = (nrows + m.G - 1) / m.G;
         cudaError_t e;
         if (m.R2 <= 16) {
             if ((e = allow_smem<k_mix2_x_inv<T, 16>>(sm)) != cudaSuccess) return e;
@@ -326,7 +328,8 @@ cudaError_t MixedPasses<T>::x_inv(int L, const C *in, int64_t in_rs, int nrows, 
     const size_t sm = gen_io_buffers(g.n, true) * swsize(L * g.TC) * sizeof(C);
     cudaError_t e = allow_smem<k_gen_x_inv<T>>(sm);
     if (e != cudaSuccess) return e;
-    k_gen_x_inv<T><<<(nrows + g.TC - 1) / g.TC, kGenThreads, sm, st>>>(in, in_rs, nrows, nvalid, o, twx, g);
+    grid = (nrows + g.TC - 1) / g.TC;
+    k_gen_x_inv<T><<<grid, kGenThreads, sm, st>>>(in, in_rs, nrows, nvalid, o, twx, g);
     return cudaGetLastError();
 }
 

@@ -80,13 +80,14 @@ cudaError_t x_fwd_pipe(const XIn<T> &a, int nrows, int nvalid, typename Cplx<T>:
 
 template <typename T, int L, bool P1>
 cudaError_t x_inv_pipe(const typename Cplx<T>::type *in, int in_rs, int nrows, int nvalid, const XOut<T> &o,
-                       const typename Cplx<T>::type *twx, cudaStream_t st)
+                       const typename Cplx<T>::type *twx, cudaStream_t st, int &grid)
 {
     using S = XShape<T, L>;
     const size_t sm = xinv_slot_bytes<T, L>(in_rs) + sizeof(uint64_t);
     cudaError_t e = allow_smem<k_x_inv_bulk<T, L, P1>>(sm);
     if (e != cudaSuccess) return e;
-    k_x_inv_bulk<T, L, P1><<<(nrows + S::TR - 1) / S::TR, S::NT, sm, st>>>(in, in_rs, nrows, nvalid, o, twx);
+    grid = (nrows + S::TR - 1) / S::TR;
+    k_x_inv_bulk<T, L, P1><<<grid, S::NT, sm, st>>>(in, in_rs, nrows, nvalid, o, twx);
     return cudaGetLastError();
 }
 }  // namespace
@@ -608,11 +609,11 @@ static bool x_inv_narrow(int L, int nrows)
 }
 
 template <typename T>
-int Passes<T>::x_blocks(int L, int nrows, int variant)
+int Passes<T>::x_blocks(int L, int nrows)
 {
     if (!pow2_len(L)) return MixedPasses<T>::x_blocks(L, nrows);
     int rows_per_cta;
-    const bool nw = x_inv_narrow<T>(L, nrows) && !(variant == 2 && L >= 64);
+    const bool nw = x_inv_narrow<T>(L, nrows);
     switch (L) {
     case 16: rows_per_cta = nw ? XShape<T, 16, 32>::TR : XShape<T, 16>::TR; break;
     case 32: rows_per_cta = nw ? XShape<T, 32, 32>::TR : XShape<T, 32>::TR; break;
@@ -627,16 +628,18 @@ int Passes<T>::x_blocks(int L, int nrows, int variant)
 
 template <typename T>
 cudaError_t Passes<T>::x_inv(int L, const C *in, int64_t in_rs, int nrows, int nvalid, const XOut<T> &o,
-                             const C *twx, cudaStream_t st, int variant)
+                             const C *twx, cudaStream_t st, int variant, int *blocks)
 {
+    int unused, &grid = blocks ? *blocks : unused;
+    grid = 0;
     if (nrows <= 0) return cudaSuccess;
-    if (!pow2_len(L)) return MixedPasses<T>::x_inv(L, in, in_rs, nrows, nvalid, o, twx, st);
+    if (!pow2_len(L)) return MixedPasses<T>::x_inv(L, in, in_rs, nrows, nvalid, o, twx, st, &grid);
     if (variant == 2 && L >= 64 && in_rs % 2 == 0 && in_rs <= 2 * L && nvalid <= L + 1 && ((uintptr_t)in & 15) == 0) {
         const bool p1 = nvalid > L;
 #define DEMAG_PIPE(LL)                                                                         \
     case LL:                                                                                   \
-        return p1 ? x_inv_pipe<T, LL, true>(in, (int)in_rs, nrows, nvalid, o, twx, st)         \
-                  : x_inv_pipe<T, LL, false>(in, (int)in_rs, nrows, nvalid, o, twx, st);
+        return p1 ? x_inv_pipe<T, LL, true>(in, (int)in_rs, nrows, nvalid, o, twx, st, grid)   \
+                  : x_inv_pipe<T, LL, false>(in, (int)in_rs, nrows, nvalid, o, twx, st, grid);
         switch (L) { DEMAG_PIPE(64) DEMAG_PIPE(128) DEMAG_PIPE(256) DEMAG_PIPE(512) default: break; }
 #undef DEMAG_PIPE
     }
@@ -646,7 +649,7 @@ cudaError_t Passes<T>::x_inv(int L, const C *in, int64_t in_rs, int nrows, int n
     if (L == LL) {                                                                             \
         using S = XShape<T, LL, 32>;                                                           \
         const size_t sm = (size_t)S::TR * S::RS * sizeof(C);                                   \
-        const int grid = (nrows + S::TR - 1) / S::TR;                                          \
+        grid = (nrows + S::TR - 1) / S::TR;                                                    \
         if (nvalid <= LL) k_x_inv2<T, LL, false, false, 32><<<grid, 32, sm, st>>>(in, in_rs, nrows, nvalid, o, twx); \
         else if (nvalid == LL + 1) k_x_inv2<T, LL, true, false, 32><<<grid, 32, sm, st>>>(in, in_rs, nrows, nvalid, o, twx); \
         else return cudaErrorInvalidValue;                                                     \
@@ -659,7 +662,7 @@ cudaError_t Passes<T>::x_inv(int L, const C *in, int64_t in_rs, int nrows, int n
     case LL: {                                                                                 \
         using S = XShape<T, LL>;                                                               \
         const size_t sm = (size_t)S::TR * S::RS * sizeof(C);                                   \
-        const int grid = (nrows + S::TR - 1) / S::TR;                                          \
+        grid = (nrows + S::TR - 1) / S::TR;                                                    \
         if (o.partials && o.Mref && nvalid <= LL && nvalid % (16 / sizeof(T)) == 0 &&          \
             o.out_rs % (16 / sizeof(T)) == 0 && ((uintptr_t)o.Mref & 15) == 0) {               \
             const size_t smp = sm + (size_t)S::TR * LL * sizeof(T);                            \
@@ -680,7 +683,7 @@ cudaError_t Passes<T>::x_inv(int L, const C *in, int64_t in_rs, int nrows, int n
         const size_t sm = swsize(LL * S::TC) * sizeof(C);                                     \
         cudaError_t e = allow_smem<k_x_inv<T, LL>>(sm);                                       \
         if (e != cudaSuccess) return e;                                                       \
-        const int grid = (nrows + S::TC - 1) / S::TC;                                         \
+        grid = (nrows + S::TC - 1) / S::TC;                                                   \
         k_x_inv<T, LL><<<grid, S::NT, sm, st>>>(in, in_rs, nrows, nvalid, o, twx);            \
         return cudaGetLastError();                                                            \
     }

@@ -49,7 +49,7 @@ template <typename T> struct MixedPasses {
     static cudaError_t x_fwd(int L, const XIn<T> &a, int nrows, int nvalid, C *out, int64_t out_rs, const C *twx,
                              cudaStream_t st);
     static cudaError_t x_inv(int L, const C *in, int64_t in_rs, int nrows, int nvalid, const XOut<T> &o,
-                             const C *twx, cudaStream_t st);
+                             const C *twx, cudaStream_t st, int *blocks);
     static int x_blocks(int L, int nrows);
     static cudaError_t col(int L, bool inv, const C *in, C *out, int ncols, int width, int64_t iss, int64_t irs,
                            int nin, int64_t oss, int64_t ors, int nout, const C *tw, int twstride, cudaStream_t st);
@@ -73,13 +73,14 @@ template <typename T> struct Passes {
     // inverse pass too; otherwise the one-tile-per-CTA kernels
     static cudaError_t x_fwd(int L, const XIn<T> &a, int nrows, int nvalid, C *out, int64_t out_rs,
                              const C *twx, cudaStream_t st, int variant = 0);
-    // complex-to-real along x with the XOut epilogue
+    // complex-to-real along x with the XOut epilogue; *blocks: the CTAs launched, each of
+    // which left one energy partial
     static cudaError_t x_inv(int L, const C *in, int64_t in_rs, int nrows, int nvalid, const XOut<T> &o,
-                             const C *twx, cudaStream_t st, int variant = 0);
+                             const C *twx, cudaStream_t st, int variant = 0, int *blocks = nullptr);
     // 1 if a bounded wait of a pipelined pass gave up since the last call (clears it)
     static int pipe_error_take();
-    // CTAs (energy partials) of the inverse x pass; the largest is variant 0's
-    static int x_blocks(int L, int nrows, int variant = 0);
+    // the most CTAs (energy partials) a form of the inverse x pass launches
+    static int x_blocks(int L, int nrows);
     // strided column transforms (y passes, z forward of the setup)
     static cudaError_t col(int L, bool inv, const C *in, C *out, int ncols, int width, int64_t iss,
                            int64_t irs, int nin, int64_t oss, int64_t ors, int nout, const C *tw,
