@@ -335,6 +335,10 @@ k_tg_field(const T *__restrict__ phi, int nx, int ny, int nz, T hx, T hy, T hz, 
                     }
             }
             if (partials) {
+                // the twelve terms of the four cells first: the chain of FP32 additions
+                // grows by one per cell column of a group, not by its terms (an FP64 sum, or
+                // sums that outlive the column in more registers, cost 13 us of 124)
+                T cell = 0;
 #pragma unroll
                 for (int p = 0; p < 3; ++p) {
                     T m4[JR];
@@ -349,8 +353,9 @@ k_tg_field(const T *__restrict__ phi, int nx, int ny, int nz, T hx, T hy, T hz, 
                         for (int q = 0; q < JR; ++q) m4[q] += ww.v[q] * x;
                     }
 #pragma unroll
-                    for (int q = 0; q < JR; ++q) acc -= m4[q] * d[q][p];
+                    for (int q = 0; q < JR; ++q) cell -= m4[q] * d[q][p];
                 }
+                acc += cell;
             }
         }
     }
