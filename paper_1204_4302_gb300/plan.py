@@ -12,6 +12,16 @@ import torch
 from . import binding as B
 
 
+def _stream_getter(c):
+    # the raw handle without a Stream object saves 2 us of a 20 us call on a small grid;
+    # the call is private to PyTorch, so where a version lacks it the public one serves
+    raw = getattr(c, "_cuda_getCurrentRawStream", None)
+    return raw if raw is not None else lambda index: torch.cuda.current_stream(index).cuda_stream
+
+
+_current_stream = _stream_getter(torch._C)
+
+
 class Plan:
     """Stray field of an nx x ny x nz grid of cells with edges (dx, dy, dz).
 
@@ -64,8 +74,7 @@ class Plan:
 
     # ------------------------------------------------------------------ basics
     def _stream(self) -> int:
-        # the raw handle without a Stream object: 2 us of a 20 us call on a small grid
-        return torch._C._cuda_getCurrentRawStream(self.device.index)
+        return _current_stream(self.device.index)
 
     def _field_arg(self, t: torch.Tensor, name: str) -> torch.Tensor:
         if not isinstance(t, torch.Tensor) or t.device != self.device:
