@@ -488,7 +488,7 @@ demag_status demag_tune_padding(int nx, int ny, int nz, double dx, double dy, do
  *    (z length 512, at most 256 input rows), 7 = as 6 with 4-column tiles and
  *    two CTAs per SM, 8 = an 8-point second stage (z lengths 32..128): FP64,
  *    variant 0 with half the registers and shared memory and two CTAs per SM;
- *    FP32, small tiles of 64 to 128 threads that read the tile-ordered tensor
+ *    FP32, small tiles of 32 to 128 threads that read the tile-ordered tensor
  *    copy, several CTAs per SM.
  *    SP plans have one form per length, and 5 (lengths 32..256); FP32 SP plans of
  *    z length 256 and 512 run persistent TMA-fed tiles whatever the variant.

@@ -98,7 +98,7 @@ template <int PASS, int L> constexpr int batch_threads()
 // the loads in flight (five CTAs of at most 48 registers; the x inverse pass keeps four).
 template <int PASS, int L> constexpr int batch_min_ctas()
 {
-    if constexpr (kBatchZt<PASS, L>) return 512 / batch_threads<PASS, L>();
+    if constexpr (kBatchZt<PASS, L>) return ZtShape<L, kBatchZC<L>>::MIN_CTAS;
     else if constexpr ((PASS == 0 && L <= 256) || ((PASS == 1 || PASS == 3) && L <= 256)) return 5;
     else if constexpr (PASS == 4 && L <= 256) return 4;
     else return 1;

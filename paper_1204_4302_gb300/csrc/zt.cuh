@@ -3,9 +3,11 @@
 // (as k_z_conv2), one small CTA per tile of TC columns kx of one ky row.
 //
 // What bounds it is the instructions per point and the latency between its
-// barriers, so the tile is small (about 1024 points a component, 64 to 128 threads,
-// some 37 KB of shared memory: 16 warps per SM in four to eight CTAs whose phases interleave), L = R1 x 8
-// is a compile-time pair, a row of the tile is a whole 64- to 256-byte segment
+// barriers, so the tile is small and several CTAs per SM interleave their phases
+// (points a component, threads, shared memory, CTAs and warps per SM: L = 32, 16 columns
+// 512, 64, 19 KB, 8, 16; 8 columns 256, 32, 11 KB, 16, 16; L = 64, 8 columns 512, 64, 20 KB,
+// 8, 16; L = 128, 16 columns 2048, 128, 73 KB, 3, 12; 8 columns 1024, 64, 38 KB, 5, 10),
+// L = R1 x 8 is a compile-time pair, a row of the tile is a whole 64- to 256-byte segment
 // (conflict-free exchange without a swizzle), the tensor block arrives from the
 // tile-ordered copy by 16-byte asynchronous copies while stage 1 runs, and the
 // product's terms are packed FP32x2 multiply-adds. Against the two-stage kernel with an
@@ -33,7 +35,11 @@ template <int L, int TC> struct ZtShape {
     static constexpr int HZ = L / 2 + 1, NSUB = TC / 4;
     static constexpr int TZB = 24 * HZ, TZS = TZB + (128 / TC - TZB % 32 + 64) % 32;
     static constexpr size_t SMEM = (size_t)3 * EXS * sizeof(float2) + (size_t)NSUB * TZS * sizeof(float);
-    static constexpr int MIN_CTAS = 512 / NT;
+    // 16 warps per SM, or what the shared memory (with a reserved kilobyte per CTA and the
+    // static sums) admits: 3 or 5 at L = 128, where asking for 4 or 8 changed nothing
+    // (128 x 128 x 64: 43.0 us)
+    static constexpr int FIT = (int)(228 * 1024 / (SMEM + 1024 + NT * sizeof(double)));
+    static constexpr int MIN_CTAS = 512 / NT < FIT ? 512 / NT : FIT;
     static_assert((R2 * TC) % NT == 0 && (R1 * TC) % NT == 0, "whole rounds of butterflies");
     static_assert(TZS % 4 == 0, "16-byte copies");
 };
