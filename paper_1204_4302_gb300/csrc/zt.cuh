@@ -50,7 +50,9 @@ enum ZtMode { ZT_FIELD = 0, ZT_ENERGY = 1, ZT_BOTH = 2 };
 
 // One tile by NT threads: the CTA, or with GRP one of its 256 / NT thread groups
 // (each group a tile of its own in its own slice of shared memory, its barriers
-// named barriers 1 + group, so the persistent batch kernel runs the same tiles).
+// named barriers 1 + group, so the persistent batch kernel runs the same tiles; the
+// spectrum, which other CTAs of that launch wrote, is then read past L1 as in its
+// other passes, ldp).
 // ntile: the tile-ordered tensor copy (zws_ntx4(Kx) sub-blocks per ky
 // row). ZT_ENERGY: nothing is written back, the CTA's part of the spectral energy
 // sum_k w(kx) m^H N^ m goes to partials[tile]; ZT_BOTH: the field and that sum,
@@ -111,7 +113,7 @@ __device__ __forceinline__ void zt_tile(float2 *__restrict__ S, int Kx, int Py, 
 #pragma unroll
             for (int r = 0; r < H1; ++r) {
                 u[i][r] = make_float2(0.f, 0.f);
-                if (ok && j + r * R2 < nrows) u[i][r] = p[(int64_t)r * R2 * rs];
+                if (ok && j + r * R2 < nrows) u[i][r] = ldp<GRP>(p + (int64_t)r * R2 * rs);
             }
         }
 #pragma unroll
