@@ -83,29 +83,34 @@ __global__ void k_tg_tables(const double *__restrict__ snode, int R, int nx, int
 // Factor transforms: on axis q, out[v][i] = sum_j D[i - j] u[v][j] for the
 // vectors v = (l, p, m) (3 R r_q of them), D the plain table (p != q) or the odd one
 // (p = q) of node l. On axis x the weight W_l lam_m^(p) / (4 pi) is folded in.
-// One launch for the three axes, a block per (l, p) and axis: its r vectors share
-// the table in shared memory, VC of them at a time with their factors as [j][VC].
-// What bounds it is shared-memory reads per multiply-add, so a thread forms
-// kTgNO outputs (a block's width apart: consecutive lanes read consecutive table
-// entries) of the VC vectors: kTgNO table reads and VC / 4 vector reads for
-// kTgNO VC multiply-adds. Rank 8 at 256^3: three launches of one output per thread (9
-// reads for 8 multiply-adds) took 70 us, this one about 45.
-constexpr int kTgNO = 4;
+// A block per (l, p) and axis: its r vectors share the table in shared memory, VC
+// of them at a time with their factors as [j][VC].
+// FP32: shared-memory reads per multiply-add bound it, so a thread forms NO = 4
+// outputs (a block's width apart: consecutive lanes read consecutive table
+// entries) of the VC vectors, NO table reads and VC / 4 vector reads for NO VC
+// multiply-adds, in one launch for the three axes. Rank 8 at 256^3: three launches of one
+// output per thread (9 reads for 8 multiply-adds) took 70 us, this one about 45.
+// FP64: the multiply-adds bound it, so none is spent on padding: one output per
+// thread, a launch per axis with its own row and rank (64^3, rank 8: 146 us, 254 in the
+// FP32 form; 64 x 48 x 200, Tucker ranks 2, 8, 16: 1417, 2190).
+template <typename T> constexpr int kTgNO = sizeof(T) == 4 ? 4 : 1;
 template <typename T> struct TgAxes {
     const T *U[3];
     T *out[3];
     int n[3], r[3];
 };
 
+// The axes q0 .. q0 + gridDim.y - 1.
 template <typename T, int VC>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(sizeof(T) == 4 ? 128 : 512)
 k_tg_apply(const T *__restrict__ tab, int tstride, const T *__restrict__ lam, const double *__restrict__ wnode, int R,
-           const TgAxes<T> ax)
+           const TgAxes<T> ax, int q0)
 {
+    constexpr int NO = kTgNO<T>;
     constexpr int W = VC < 4 ? VC : 4;  // values per vector read
     struct alignas(W * sizeof(T) < 16 ? W * sizeof(T) : 16) Vec { T v[W]; };
     extern __shared__ __align__(16) unsigned char smraw[];
-    const int q = blockIdx.y, n = ax.n[q], r = ax.r[q];
+    const int q = q0 + blockIdx.y, n = ax.n[q], r = ax.r[q];
     const T *__restrict__ U = ax.U[q];
     T *__restrict__ out = ax.out[q];
     T *su = reinterpret_cast<T *>(smraw);   // [n][VC]
@@ -127,11 +132,11 @@ k_tg_apply(const T *__restrict__ tab, int tstride, const T *__restrict__ lam, co
                                               (1.0 / (4.0 * 3.14159265358979323846)))
                                         : (T)1;
         __syncthreads();
-        for (int i0 = threadIdx.x; i0 < n; i0 += kTgNO * blockDim.x) {
-            T acc[kTgNO][VC];
-            const T *d[kTgNO];
+        for (int i0 = threadIdx.x; i0 < n; i0 += NO * blockDim.x) {
+            T acc[NO][VC];
+            const T *d[NO];
 #pragma unroll
-            for (int o = 0; o < kTgNO; ++o) {
+            for (int o = 0; o < NO; ++o) {
                 // an output past the row reads the last one's table entries and is dropped
                 d[o] = st + min(i0 + o * (int)blockDim.x, n - 1) + n - 1;
 #pragma unroll
@@ -146,14 +151,14 @@ k_tg_apply(const T *__restrict__ tab, int tstride, const T *__restrict__ lam, co
                     for (int e = 0; e < W; ++e) f[h * W + e] = w.v[e];
                 }
 #pragma unroll
-                for (int o = 0; o < kTgNO; ++o) {
+                for (int o = 0; o < NO; ++o) {
                     const T dv = d[o][-j];
 #pragma unroll
                     for (int mm = 0; mm < VC; ++mm) acc[o][mm] += dv * f[mm];
                 }
             }
 #pragma unroll
-            for (int o = 0; o < kTgNO; ++o) {
+            for (int o = 0; o < NO; ++o) {
                 const int i = i0 + o * (int)blockDim.x;
                 if (i >= n) continue;
                 for (int mm = 0; mm < mc; ++mm) {
@@ -164,21 +169,40 @@ k_tg_apply(const T *__restrict__ tab, int tstride, const T *__restrict__ lam, co
     }
 }
 
+// The launch of axes q0 .. q0 + nq - 1.
 template <typename T>
-cudaError_t tg_apply(const T *tab, int tstride, const TgAxes<T> &ax, const T *lam, const double *wnode, int R, cudaStream_t st)
+cudaError_t tg_apply_axes(const T *tab, int tstride, const TgAxes<T> &ax, const T *lam, const double *wnode, int R, int q0, int nq,
+                          cudaStream_t st)
 {
-    const int n = std::max(ax.n[0], std::max(ax.n[1], ax.n[2])), r = std::max(ax.r[0], std::max(ax.r[1], ax.r[2]));
-    const int threads = std::min(128, (n + 32 * kTgNO - 1) / (32 * kTgNO) * 32);
+    constexpr int NO = kTgNO<T>;
+    const int n = *std::max_element(ax.n + q0, ax.n + q0 + nq), r = *std::max_element(ax.r + q0, ax.r + q0 + nq);
+    const int threads = std::min(sizeof(T) == 4 ? 128 : 512, (n + 32 * NO - 1) / (32 * NO) * 32);
     const int vc = r >= 8 ? 8 : (r >= 4 ? 4 : (r >= 2 ? 2 : 1));
     const size_t sm = (size_t)(vc * n + 2 * n) * sizeof(T);
-    const dim3 grid(3 * R, 3);
+    const dim3 grid(3 * R, nq);
     switch (vc) {
-    case 8: k_tg_apply<T, 8><<<grid, threads, sm, st>>>(tab, tstride, lam, wnode, R, ax); break;
-    case 4: k_tg_apply<T, 4><<<grid, threads, sm, st>>>(tab, tstride, lam, wnode, R, ax); break;
-    case 2: k_tg_apply<T, 2><<<grid, threads, sm, st>>>(tab, tstride, lam, wnode, R, ax); break;
-    default: k_tg_apply<T, 1><<<grid, threads, sm, st>>>(tab, tstride, lam, wnode, R, ax); break;
+    case 8: k_tg_apply<T, 8><<<grid, threads, sm, st>>>(tab, tstride, lam, wnode, R, ax, q0); break;
+    case 4: k_tg_apply<T, 4><<<grid, threads, sm, st>>>(tab, tstride, lam, wnode, R, ax, q0); break;
+    case 2: k_tg_apply<T, 2><<<grid, threads, sm, st>>>(tab, tstride, lam, wnode, R, ax, q0); break;
+    default: k_tg_apply<T, 1><<<grid, threads, sm, st>>>(tab, tstride, lam, wnode, R, ax, q0); break;
     }
     return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t tg_apply(const T *tab, int tstride, const TgAxes<T> &ax, const T *lam, const double *wnode, int R, long &launches,
+                     cudaStream_t st)
+{
+    if (sizeof(T) == 4) {
+        ++launches;
+        return tg_apply_axes<T>(tab, tstride, ax, lam, wnode, R, 0, 3, st);
+    }
+    cudaError_t e = cudaSuccess;
+    for (int q = 0; q < 3 && e == cudaSuccess; ++q) {
+        e = tg_apply_axes<T>(tab, tstride, ax, lam, wnode, R, q, 1, st);
+        ++launches;
+    }
+    return e;
 }
 
 // Dense block-CP contraction Phi[k][j][i] = sum_K Z[K][k] Y[K][j] X[K][i].
@@ -524,9 +548,8 @@ demag_status tg_run(demag_tg_plan *p, const void *lam, const void *Ux, const voi
         ax.n[q] = n[q];
         ax.r[q] = rq[q];
     }
-    cudaError_t ea = tg_apply<T>(static_cast<const T *>(p->tab), p->tstride, ax, weights, p->wnode, p->R, st);
+    cudaError_t ea = tg_apply<T>(static_cast<const T *>(p->tab), p->tstride, ax, weights, p->wnode, p->R, p->launches, st);
     if (ea != cudaSuccess) return tg_fail(DEMAG_ERR_CUDA, std::string("TG factor transforms: ") + cudaGetErrorString(ea));
-    p->launches++;
     const bool mma = std::is_same<T, float>::value && p->contraction == 1;
     if (p->tucker) {
         const dim3 grid(3 * p->R, p->nz);
