@@ -499,7 +499,7 @@ demag_status demag_tune_padding(int nx, int ny, int nz, double dx, double dy, do
  *    512 and 1024), 3 = as 2, with the forward pass by persistent CTAs that
  *    receive their column tiles by TMA tensor copies (two tiles in flight).
  *    FP32 plans have one form at y lengths 512 and 1024, whatever the variant;
- *    an FP64 plan that is not autotuned starts with 2 there, else 0.
+ *    an FP64 plan that is not autotuned starts with 2 at 512, else 0.
  *    A variant that does not exist for the plan's lengths runs as variant 0.
  *    Out-of-range values: DEMAG_ERR_INVALID_ARG. */
 demag_status demag_get_variants(demag_plan_t plan, int *z, int *y);

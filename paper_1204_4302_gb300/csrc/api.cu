@@ -767,7 +767,9 @@ int sp_smooth_pad(int n)
 // Kernel forms of a plan that is not autotuned, by the lengths alone: the ones
 // the autotuner keeps almost everywhere at these lengths (FP32 fields, ms, this form
 // against the two-stage forms of variant 0: z pass at 256^3 0.63 / 1.08, 128^3 0.070 /
-// 0.155, 64^3 0.018 / 0.027, 16^3 0.008 / 0.026; FP64 z pass at 64^3 0.30 / 0.36).
+// 0.155, 64^3 0.018 / 0.027, 16^3 0.008 / 0.026; FP64 z pass at 64^3 0.30 / 0.36; FP64
+// y form 2 against 0, whole field: y length 512 64 x 200 x 20 0.84 / 0.85, 30 x 256 x 16
+// 0.319 / 0.326, but 1024 512 x 512 x 1 0.49 / 0.43, 40 x 512 x 40 3.72 / 3.65).
 void default_variants(demag_plan *p, int method, demag_prec prec, const int P[3])
 {
     const bool dm32 = method == DEMAG_METHOD_DM && prec == DEMAG_F32;
@@ -775,7 +777,7 @@ void default_variants(demag_plan *p, int method, demag_prec prec, const int P[3]
     p->xvariant = prec == DEMAG_F32 ? 2 : 1;  // bulk-copy x passes where the rows allow them
     if (dm32 && (L == 256 || L == 512)) p->zvariant = 6;
     else if (method == DEMAG_METHOD_DM && (L == 32 || L == 64 || L == 128)) p->zvariant = 8;
-    if (prec == DEMAG_F64 && (P[1] == 512 || P[1] == 1024)) p->yvariant = 2;  // FP32 has one form there
+    if (prec == DEMAG_F64 && P[1] == 512) p->yvariant = 2;  // FP32 has one form there
 }
 
 // Allocates a plan with padded lengths P for the given method (no launches).
