@@ -801,7 +801,9 @@ cudaError_t Passes<T>::col(int L, bool inv, const C *in, C *out, int ncols, int 
                                              : col_launch<LL, true, false, true, 0>(in, out, ncols, width, iss, irs, nin, oss, ors, nout, tw, twstride, st); \
         if (inv) return col_launch<LL, true, false, false, 0>(in, out, ncols, width, iss, irs, nin, oss, ors, nout, tw, twstride, st); \
         return col_launch<LL, false, false, false, 0>(in, out, ncols, width, iss, irs, nin, oss, ors, nout, tw, twstride, st);
-    switch (L) { DEMAG_CASE(32) DEMAG_CASE(64) DEMAG_CASE(128) DEMAG_CASE(256) DEMAG_CASE(512) DEMAG_CASE(1024) default: return cudaErrorInvalidValue; }
+    if constexpr (sizeof(T) == 8)  // FP32 columns of these lengths are the pruned field passes above
+        switch (L) { DEMAG_CASE(512) DEMAG_CASE(1024) default: break; }
+    switch (L) { DEMAG_CASE(32) DEMAG_CASE(64) DEMAG_CASE(128) DEMAG_CASE(256) default: return cudaErrorInvalidValue; }
 #undef DEMAG_CASE
 }
 
