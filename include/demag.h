@@ -137,9 +137,10 @@ typedef struct {
     double dx, dy, dz;       /* cell edges */
     int energy_in_z;         /* 1: a field call with the energy takes the
                                 energy's spectral sum in its z pass (FP32
-                                plan, persistent z form, z length 256 or 512,
-                                spectral route on), so its last pass does not
-                                read M; 0: the last pass sums M.H */
+                                plan, z form 6 or 7 at z length 256 or 512 or
+                                form 8 at 32 to 128, spectral route on), so
+                                its last pass does not read M; 0: the last
+                                pass sums M.H */
 } demag_info;
 
 /* Create a plan for an nx x ny x nz grid with cell edges dx, dy, dz.
@@ -250,8 +251,8 @@ demag_status demag_energy(demag_plan_t plan, const void *M, double *E_out, void 
  * spectral sum where the plan allows it, 0 always runs the field pipeline.
  * Both give E within rounding; the spectral route skips the y and x inverse
  * passes. The same switch decides whether field calls with the energy take
- * the spectral sum in the persistent z pass (demag_info.energy_in_z) or the
- * sum of M.H in their last pass. Tensor-method plans only (scalar-potential
+ * the spectral sum in the z pass (where demag_info.energy_in_z can be 1) or
+ * the sum of M.H in their last pass. Tensor-method plans only (scalar-potential
  * plans always run their own pipeline). */
 demag_status demag_set_spectral_energy(demag_plan_t plan, int enable);
 

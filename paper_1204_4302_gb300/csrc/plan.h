@@ -68,9 +68,9 @@ template <typename T> struct MixedPasses {
 template <typename T> struct Passes {
     using C = typename CplxOf<T>::type;
     // real-to-complex along x; L = Px/2 (complex length), Px >= 2
-    // variant 1: the forward pass by persistent CTAs streaming row tiles
-    // with bulk asynchronous copies (where the rows allow it); variant 2: the
-    // inverse pass too; otherwise the one-tile-per-CTA kernels
+    // variant >= 1, FP64: persistent CTAs streaming row tiles with bulk
+    // asynchronous copies (where the rows allow it); otherwise one tile per CTA.
+    // x_inv, variant 2: a tile's rows arrive by one bulk copy
     static cudaError_t x_fwd(int L, const XIn<T> &a, int nrows, int nvalid, C *out, int64_t out_rs,
                              const C *twx, cudaStream_t st, int variant = 0);
     // complex-to-real along x with the XOut epilogue; *blocks: the CTAs launched, each of

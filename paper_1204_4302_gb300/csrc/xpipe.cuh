@@ -1,10 +1,11 @@
-// Pipelined x passes: persistent CTAs stream their tiles of whole rows
-// through shared memory with bulk asynchronous copies (TMA, cp.async.bulk)
-// completing on mbarriers, two tiles in flight per CTA, so the loads of the
-// next tiles overlap the transforms of the current one. Same arithmetic and
-// results as k_x_fwd2 / k_x_inv2; used when the tile's rows are contiguous
-// and 16-byte multiples (the field passes of plans with nx % 4 == 0 for the
-// forward pass; always for the inverse pass, whose rows are Kxp complex).
+// x passes whose tiles of whole rows arrive by bulk asynchronous copies (TMA,
+// cp.async.bulk) completing on mbarriers. Forward (FP64): persistent CTAs, two tiles
+// in flight each, so the loads of the next tiles overlap the transforms of the
+// current one. Inverse: one tile per CTA, several CTAs per SM overlap. Same
+// arithmetic and results as k_x_fwd2 / k_x_inv2; used when the tile's rows are
+// contiguous and 16-byte multiples (the field passes of plans with nx % 4 == 0 for
+// the forward pass; always for the inverse pass, whose rows are Kxp complex). The
+// FP64 y forward pass by TMA tensor copies is here too.
 #pragma once
 #include <cuda.h>  // CUtensorMap (the map is built on the host, see passes_impl.cuh)
 
