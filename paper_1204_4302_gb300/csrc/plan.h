@@ -224,8 +224,8 @@ struct demag_plan {
     // tensor spectrum [6][Pz/2+1][Py/2+1][Kx] (SP: kernel tables [3][...])
     double *nhat64;
     float *nhat32;
-    // tile-ordered copy of nhat32 for the persistent TMA z pass (z variant 6;
-    // FP32 tensor-method plans whose z length it supports), else null
+    // tile-ordered copy of nhat32 for the z passes that read it (build_ntile); null for
+    // other lengths, and where memory ran out
     float *ntile;
     size_t ntile_bytes;
     // SP: half-sample phase factors exp(-pi i k / P) per axis, k < P
