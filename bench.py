@@ -1269,7 +1269,7 @@ def main():
     args = ap.parse_args()
     if args.write_traffic:
         write_traffic(args.write_traffic, args.traffic_command,
-                      "256^3 FP32 field + energy, padded 512^3, z variant 6, y 2, x 1")
+                      "256^3 FP32 field + energy, padded 512^3, z variant 6, y 0, x 2")
         return
     if args.warmup < 3:
         args.warmup = 3
